@@ -34,6 +34,8 @@ static __constant__ double c_E[4][3][18] = {
     {RLBM_E_MJ_INIT, RLBM_E_FD_INIT, RLBM_E_BE_INIT}};
 constexpr int kOrder5 = 3;  // table index of the fifth order
 static __constant__ double c_pnk[63] = RLBM_PNK_INIT;
+static __constant__ double c_logser[5 * RLBM_NLOGSER] = RLBM_LOGSER_INIT;
+static __constant__ double c_rev[RLBM_NREV] = RLBM_REV_INIT;
 static __constant__ double c_invpow[6 * RLBM_NSERIES] = RLBM_INVPOW_INIT;
 static __constant__ double c_be_exp[6 * RLBM_NEXP] = RLBM_BE_EXP_INIT;
 static __constant__ double c_fd_exp[6 * RLBM_NEXP] = RLBM_FD_EXP_INIT;
@@ -43,6 +45,35 @@ static __constant__ double c_g_zc[6] = RLBM_G_ZC_INIT;
 
 // Offset of harmonic block k in the Q tables: sum_{k'<k} 6 (6 - k').
 __host__ __device__ constexpr int qoff(int k) { return 6 * (6 * k - (k * (k - 1)) / 2); }
+
+// Moment polynomials P_nk(u^2) (Appendix), entry 3 * (n(n+1)/2 + k) + power: a
+// compile-time function, so that the 42 coefficients that are 0 cost nothing.
+__host__ __device__ constexpr double pnk(int i) {
+  constexpr double t[63] = RLBM_PNK_INIT;
+  return t[i];
+}
+
+// ------------------------------------------------ FP64 divide and square root
+// GB300 issues one FP64 warp instruction per SM sub-partition every 64 clocks, so a
+// reciprocal or a root costs what its FP64 instructions cost. Both start from the
+// FP32 unit's value (about 24 bits) and take one step of a third-order (Halley)
+// iteration in FP64: with e = 1 - x r, 1/x = r (1 + e + e^2 + ...), and with
+// e = 1 - x r^2, 1/sqrt(x) = r (1 + e/2 + 3 e^2/8 + ...); the terms left out are
+// below 2^-66. Outside the FP32 range they fall back to the compiler's own.
+__device__ __forceinline__ double rcp64(double x) {
+  const float xf = (float)x;
+  if (!(fabsf(xf) > 1e-30f && fabsf(xf) < 1e30f)) return 1.0 / x;
+  const double r = (double)(1.0f / xf);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double rsqrt64(double x) {
+  const float xf = (float)x;
+  if (!(xf > 1e-30f && xf < 1e30f)) return 1.0 / sqrt(x);
+  const double r = (double)rsqrtf(xf);
+  const double e = fma(-(x * r), r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
 
 // ------------------------------------------------------- EDF integrals g_nu
 // g[nu-1] = g_nu(z), nu = 1..6 (Eq. 12). MJ: z. BE: Li_nu(z). FD: -Li_nu(-z).
@@ -169,7 +200,7 @@ __device__ __forceinline__ bool newton_done64(double d, double z) {
 // 1.4e-6 off in mu at z = 0.17: two Newton steps reach the FP64 floor, a third
 // confirms it.
 template <int EDF>
-__device__ int solve_z_from_R(double target, double& z, double g[6]) {
+__device__ __noinline__ int solve_z_from_R_general(double target, double& z, double g[6]) {
   if (EDF == EDF_BE && target < RLBM_R_ZC) {
     z = ZC;
 #pragma unroll
@@ -218,13 +249,8 @@ __device__ int solve_z_from_R(double target, double& z, double g[6]) {
 // G = g_2(z) gives mu = ln G +- G/4 - (5/288) G^2 +- G^3/288 + O(G^4) (upper
 // signs FD, lower BE).
 template <int EDF>
-__device__ int solve_z_from_n_theta(double n, double theta, double& z, double g[6]) {
+__device__ __noinline__ int solve_z_from_n_theta_general(double n, double theta, double& z, double g[6]) {
   const double G = n / (2.0 * PI * theta * theta);
-  if (EDF == EDF_MJ) {
-    z = G;
-    g_all<EDF>(z, g);
-    return 0;
-  }
   if (EDF == EDF_BE && G >= c_g_zc[1]) {
     z = ZC;
 #pragma unroll
@@ -268,6 +294,165 @@ __device__ int solve_z_from_n_theta(double n, double theta, double& z, double g[
   return st;
 }
 
+// Fugacity in the variable t = g_1 = ln(1 + z) (FD) or -ln(1 - z) (BE), for t up
+// to kTMax (z = 2.8 FD, 0.74 BE): there g_nu = t sum_n c_nu[n] (s t)^n (s = -1
+// FD, +1 BE) with convergence radius 2 pi, so 11 to 28 terms of five series do what
+// took 23 to 48 of six, and neither a logarithm nor an exponential is evaluated.
+constexpr float kTMax = 1.35f;
+
+// terms that put the first one left out below 2^-58 of the sum for every nu
+__device__ __forceinline__ int logser_terms(float t) { return t <= 0.2f ? 12 : (t <= 0.45f ? 16 : (t <= 0.75f ? 20 : 28)); }
+
+// g_2 and g_3 (FP32, 12 terms: 1e-7 at kTMax)
+template <int EDF>
+__device__ __forceinline__ void g23_t_f(float t, float& g2, float& g3) {
+  const float u = EDF == EDF_BE ? t : -t, u2 = u * u;
+  float a = 0.0f, b = 0.0f;
+#pragma unroll
+  for (int n = 10; n >= 2; n -= 2) a = fmaf(a, u2, (float)c_logser[n]);
+#pragma unroll
+  for (int n = 11; n >= 0; --n) b = fmaf(b, u, (float)c_logser[RLBM_NLOGSER + n]);
+  g2 = t * fmaf(a, u2, fmaf(u, -0.25f, 1.0f));
+  g3 = t * b;
+}
+
+// g_0 = z dg_1/dz (FP32): z/(1 + z) = 1 - e^-t (FD), z/(1 - z) = e^t - 1 (BE)
+template <int EDF>
+__device__ __forceinline__ float g0_t_f(float t) { return EDF == EDF_BE ? expm1f(t) : -expm1f(-t); }
+
+// g_2 (even terms beyond the second vanish, Li_2 - u + u^2/4 being odd) and g_3
+template <int EDF>
+__device__ __forceinline__ void g23_t(double t, int nt, double& g2, double& g3) {
+  const double u = EDF == EDF_BE ? t : -t, u2 = u * u;
+  double a = 0.0, b = 0.0;
+  for (int n = nt; n >= 2; n -= 2) {
+    a = fma(a, u2, c_logser[n]);
+    b = fma(fma(b, u, c_logser[RLBM_NLOGSER + n + 1]), u, c_logser[RLBM_NLOGSER + n]);
+  }
+  b = fma(fma(b, u, c_logser[RLBM_NLOGSER + 1]), u, c_logser[RLBM_NLOGSER]);
+  g2 = t * fma(a, u2, fma(u, -0.25, 1.0));
+  g3 = t * b;
+}
+
+// all six (g_1 = t)
+template <int EDF>
+__device__ __forceinline__ void g_all_t(double t, int nt, double g[6]) {
+  const double u = EDF == EDF_BE ? t : -t, u2 = u * u;
+  double a = 0.0, b[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int n = nt; n >= 2; n -= 2) {
+    a = fma(a, u2, c_logser[n]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      b[j] = fma(fma(b[j], u, c_logser[(j + 1) * RLBM_NLOGSER + n + 1]), u, c_logser[(j + 1) * RLBM_NLOGSER + n]);
+  }
+  g[0] = t;
+  g[1] = t * fma(a, u2, fma(u, -0.25, 1.0));
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    g[2 + j] = t * fma(fma(b[j], u, c_logser[(j + 1) * RLBM_NLOGSER + 1]), u, c_logser[(j + 1) * RLBM_NLOGSER]);
+}
+
+// z of t
+template <int EDF>
+__device__ __forceinline__ double z_of_t(double t) { return EDF == EDF_BE ? -expm1(-t) : expm1(t); }
+
+// g_nu moved by a step dmu of ln z that is below 1e-9: dg_nu/dmu = g_(nu-1), the
+// second-order term is below 1e-18.
+__device__ __forceinline__ void g_shift(double dmu, float g0, double g[6]) {
+#pragma unroll
+  for (int i = 5; i >= 1; --i) g[i] = fma(dmu, g[i - 1], g[i]);
+  g[0] = fma(dmu, (double)g0, g[0]);
+}
+
+// Fugacity from (eps, n), FD/BE: g_3^2/g_2^3 = target (Eq. 25). In t the ratio is
+// w = 1/target = g_2^3/g_3^2 = t - (47/1728) t^3 - ..., so the reversion gives t to
+// FP32 accuracy; one FP64 Newton step (in mu = ln z, whose F' = 2 g_2/g_3 - 3 g_1/g_2
+// may be FP32) leaves about 1e-13, and the second one, taken from the residual at
+// that point and carried to the six g_nu to first order, about 1e-20. States outside
+// the series' range, and any whose second step is not small, take the general
+// solver. kZ: z is wanted (the step only needs the g_nu).
+template <int EDF, bool kZ>
+__device__ __forceinline__ int solve_z_from_R(double target, double& z, double g[6]) {
+  const float wf = 1.0f / (float)target;
+  if (wf > 1e-20f && wf < 1.25f) {
+    const float sw = EDF == EDF_BE ? wf : -wf;
+    float p = 0.0f;
+#pragma unroll
+    for (int n = RLBM_NREV - 1; n >= 0; --n) p = fmaf(p, sw, (float)c_rev[n]);
+    float tf = wf * p;
+    if (wf > 0.5f) {  // the reversion's own series is short there: two FP32 steps
+#pragma unroll
+      for (int it = 0; it < 2; ++it) {
+        float a, b;
+        g23_t_f<EDF>(tf, a, b);
+        tf -= (a * a * a / (b * b) - wf) / fmaf(-47.0f / 576.0f, tf * tf, 1.0f);
+      }
+    }
+    if (tf > 0.0f && tf <= kTMax) {
+      const int nt = logser_terms(tf);
+      double t = (double)tf, g2, g3;
+      g23_t<EDF>(t, nt, g2, g3);
+      float g0 = g0_t_f<EDF>(tf);
+      {
+        const double a = target * (g2 * g2 * g2);
+        const float x = (float)fma(g3, g3, -a) / (float)a, r2 = (float)g2, r3 = (float)g3;
+        const float dmu = -x * fmaf(-0.5f, x, 1.0f) / (2.0f * r2 / r3 - 3.0f * tf / r2);
+        t += (double)(dmu * g0);
+      }
+      g_all_t<EDF>(t, nt, g);
+      const double a = target * (g[1] * g[1] * g[1]);
+      const float r2 = (float)g[1], r3 = (float)g[2];
+      const float dmu = -((float)fma(g[2], g[2], -a) / (float)a) / (2.0f * r2 / r3 - 3.0f * tf / r2);
+      if (fabsf(dmu) < 1e-9f) {
+        g_shift((double)dmu, g0, g);
+        if (kZ) z = z_of_t<EDF>(g[0]);
+        return 0;
+      }
+    }
+  }
+  return solve_z_from_R_general<EDF>(target, z, g);
+}
+
+// Fugacity from (n, theta): n = 2 pi theta^2 g_2(z), as solve_z_from_R with
+// G = g_2 = t + s t^2/4 + ... inverted in FP32 by Newton (dg_2/dt = t / g_0).
+template <int EDF, bool kZ>
+__device__ __forceinline__ int solve_z_from_n_theta(double n, double theta, double& z, double g[6]) {
+  const double G = n / (2.0 * PI * theta * theta);
+  if (EDF == EDF_MJ) {
+    z = G;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) g[i] = G;
+    return 0;
+  } else {
+    const float Gf = (float)G;
+    if (Gf > 1e-20f && Gf < 1.25f) {
+      float tf = Gf * fmaf(Gf, fmaf(7.0f / 72.0f, Gf, EDF == EDF_BE ? 0.25f : -0.25f), 1.0f);
+      if (EDF == EDF_BE) tf = fminf(tf, kTMax);
+#pragma unroll
+      for (int it = 0; it < 4; ++it) {
+        float a, b;
+        g23_t_f<EDF>(tf, a, b);
+        tf -= (a - Gf) * g0_t_f<EDF>(tf) / tf;
+      }
+      if (tf > 0.0f && tf <= kTMax) {
+        const int nt = logser_terms(tf);
+        double t = (double)tf, g2, g3;
+        g23_t<EDF>(t, nt, g2, g3);
+        const float g0 = g0_t_f<EDF>(tf);
+        t += (double)((float)(G - g2) * g0 / tf);
+        g_all_t<EDF>(t, nt, g);
+        const float dmu = (float)(G - g[1]) / tf;
+        if (fabsf(dmu) < 1e-9f) {
+          g_shift((double)dmu, g0, g);
+          if (kZ) z = z_of_t<EDF>(g[0]);
+          return 0;
+        }
+      }
+    }
+  }
+  return solve_z_from_n_theta_general<EDF>(n, theta, z, g);
+}
+
 // ------------------------------------------------------------ Landau frame
 // T^a_b U^b = eps U^a (Eq. 21) written for U = gamma (1, u):
 //   eps = T00 - m.u,   m_i - Pi_ij u_j = eps u_i,   m = (T01, T02), Pi = T^{ij},
@@ -276,12 +461,16 @@ __device__ int solve_z_from_n_theta(double n, double theta, double& z, double g[
 // the eigenvector the paper's power method converges to.
 struct Frame {
   double eps, ux, uy, gamma;
+  int st;
 };
 
-__device__ __forceinline__ int landau(const double T[6], Frame& F) {
-  const double E = T[0], mx = T[1], my = T[2], pxx = T[3], pxy = T[4], pyy = T[5];
+// Any state: FP64 Newton throughout.
+static __device__ __noinline__ Frame landau_general(double E, double mx, double my, double pxx, double pxy, double pyy) {
+  Frame F;
+  F.eps = F.ux = F.uy = F.gamma = 0.0;
+  F.st = ST_NONPHYSICAL;
   const double disc = 9.0 * E * E - 8.0 * (mx * mx + my * my);
-  if (!(E > 0.0) || !(disc >= 0.0)) return ST_NONPHYSICAL;
+  if (!(E > 0.0) || !(disc >= 0.0)) return F;
   const double x = 0.25 * (3.0 * E + sqrt(disc));
   double ux = mx / x, uy = my / x;
   int st = ST_LANDAU;
@@ -299,13 +488,66 @@ __device__ __forceinline__ int landau(const double T[6], Frame& F) {
     if (fmax(fabs(dx), fabs(dy)) < 1e-13) { st = 0; break; }
   }
   const double u2 = ux * ux + uy * uy;
-  if (!(u2 < 1.0)) return ST_NONPHYSICAL;
+  if (!(u2 < 1.0)) return F;
   F.ux = ux;
   F.uy = uy;
   F.eps = E - (mx * ux + my * uy);
   F.gamma = 1.0 / sqrt(1.0 - u2);
-  if (!(F.eps > 0.0)) return ST_NONPHYSICAL;
-  return st;
+  if (F.eps > 0.0) F.st = st;
+  return F;
+}
+
+// The same root with the iterations in FP32: Newton in FP32 (about 1e-7), then FP64
+// residuals corrected through the FP32 Jacobian, whose 1e-6 only scales a correction,
+// so two of them reach the FP64 floor (about 30 FP64 instructions against 270 for five
+// FP64 steps). States near the light cone or out of the
+// FP32 range, and any whose corrections do not shrink, take landau_general.
+__device__ __forceinline__ int landau(const double T[6], Frame& F) {
+  const float E = (float)T[0], mx = (float)T[1], my = (float)T[2], pxx = (float)T[3], pxy = (float)T[4],
+              pyy = (float)T[5];
+  const float disc = fmaf(9.0f * E, E, -8.0f * fmaf(mx, mx, my * my));
+  if (E > 1e-15f && E < 1e15f && disc > 0.1f * E * E) {
+    const float rx = 4.0f / fmaf(3.0f, E, sqrtf(disc));
+    float fu = mx * rx, fv = my * rx, j00, j01, j10, j11, rdet;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      const float a = fmaf(-mx, fu, fmaf(-my, fv, E));
+      j00 = fmaf(fu, mx, -pxx) - a;
+      j01 = fmaf(fu, my, -pxy);
+      j10 = fmaf(fv, mx, -pxy);
+      j11 = fmaf(fv, my, -pyy) - a;
+      rdet = 1.0f / fmaf(j00, j11, -j01 * j10);
+      if (it == 3) break;  // the Jacobian at the FP32 root
+      const float fx = fmaf(-a, fu, fmaf(-pxx, fu, fmaf(-pxy, fv, mx)));
+      const float fy = fmaf(-a, fv, fmaf(-pxy, fu, fmaf(-pyy, fv, my)));
+      fu = fmaf(fmaf(j01, fy, -j11 * fx), rdet, fu);
+      fv = fmaf(fmaf(j10, fx, -j00 * fy), rdet, fv);
+    }
+    if (fmaf(fu, fu, fv * fv) < 0.95f) {
+      double ux = (double)fu, uy = (double)fv;
+      float d = 0.0f;
+      for (int it = 0; it < 6; ++it) {
+        const double a = fma(-T[1], ux, fma(-T[2], uy, T[0]));
+        const float fx = (float)fma(-a, ux, fma(-T[3], ux, fma(-T[4], uy, T[1])));
+        const float fy = (float)fma(-a, uy, fma(-T[4], ux, fma(-T[5], uy, T[2])));
+        const float dx = fmaf(j01, fy, -j11 * fx) * rdet, dy = fmaf(j10, fx, -j00 * fy) * rdet;
+        ux += (double)dx;
+        uy += (double)dy;
+        d = fmaxf(fabsf(dx), fabsf(dy));
+        if (d < 2e-11f) break;  // the next one would be below 1e-16
+      }
+      if (d < 2e-11f) {
+        F.ux = ux;
+        F.uy = uy;
+        F.eps = fma(-T[1], ux, fma(-T[2], uy, T[0]));
+        F.gamma = rsqrt64(fma(-ux, ux, fma(-uy, uy, 1.0)));
+        if (!(F.eps > 0.0)) return ST_NONPHYSICAL;
+        return 0;
+      }
+    }
+  }
+  F = landau_general(T[0], T[1], T[2], T[3], T[4], T[5]);
+  return F.st;
 }
 
 // Macroscopic state of a cell: n = U_mu N^mu, theta, z (Eqs. 23-25).
@@ -314,8 +556,9 @@ struct CellState {
   double g[6];
 };
 
-template <int EDF>
-__device__ int cell_state(const double N[3], const double T[6], CellState& S) {
+// kZ: z is wanted (the read-out; a step only needs the g_nu).
+template <int EDF, bool kZ>
+__device__ __forceinline__ int cell_state(const double N[3], const double T[6], CellState& S) {
   Frame F;
   int st = landau(T, F);
   if (st & ST_NONPHYSICAL) return st;
@@ -323,122 +566,151 @@ __device__ int cell_state(const double N[3], const double T[6], CellState& S) {
   S.uy = F.uy;
   S.gamma = F.gamma;
   S.eps = F.eps;
-  S.n = F.gamma * (N[0] - F.ux * N[1] - F.uy * N[2]);
+  S.n = F.gamma * fma(-F.ux, N[1], fma(-F.uy, N[2], N[0]));
   if (!(S.n > 0.0) || !isfinite(S.n) || !isfinite(S.eps)) return st | ST_NONPHYSICAL;
   if (EDF == EDF_MJ) {
-    S.theta = S.eps / (2.0 * S.n);
-    S.z = S.n / (2.0 * PI * S.theta * S.theta);
+    S.theta = 0.5 * (S.eps * rcp64(S.n));
+    if (kZ) {
+      S.z = S.n / (2.0 * PI * S.theta * S.theta);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) S.g[i] = S.z;
+      for (int i = 0; i < 6; ++i) S.g[i] = S.z;
+    }
     return st;
   }
-  const double target = 0.5 * PI * S.eps * S.eps / (S.n * S.n * S.n);
-  const int zs = solve_z_from_R<EDF>(target, S.z, S.g);
+  const double rn = rcp64(S.n), en = S.eps * rn;
+  const double target = (0.5 * PI) * (en * en * rn);
+  const int zs = solve_z_from_R<EDF, kZ>(target, S.z, S.g);
   st |= zs;
   if (zs & ST_CLAMPED) S.theta = sqrt(S.n / (2.0 * PI * S.g[1]));
-  else S.theta = 0.5 * S.g[1] / S.g[2] * S.eps / S.n;
+  else S.theta = 0.5 * (S.g[1] * rcp64(S.g[2])) * en;
   return st;
 }
 
 // --------------------------------------------- equilibrium moments (harmonic)
-// Z_nk = int dp dphi f^eq p^n e^{i k phi}
-//      = 2 pi n! g_{n+1}(z) theta^{n+1} gamma^n (u_x + i u_y)^k P_nk(u^2),  k <= n <= 5.
-// zr/zi are indexed n(n+1)/2 + k. When nA1 / eA2 are non-negative they replace
-// the degree-1 and degree-2 prefactors 2 pi g_2 theta^2 = n and
-// 2 pi 2! g_3 theta^3 = eps (Eq. 25), so that the equilibrium carries the cell's
-// own n and eps exactly and the collision conserves N^0 and T^{mu 0} without a
-// rounding bias from the z, theta round trip.
+// Z_nk = int dp dphi f^eq p^n e^{i k phi} = Y_nk (u_x + i u_y)^k,
+// Y_nk = 2 pi n! g_{n+1}(z) theta^{n+1} gamma^n P_nk(u^2),  k <= n <= 5: the real
+// factors y, indexed n(n+1)/2 + k. The degree-1 and degree-2 prefactors are the
+// cell's own n gamma and eps gamma^2 (2 pi g_2 theta^2 = n, 4 pi g_3 theta^3 = eps,
+// Eq. 25), so that the collision conserves N^0 and T^{mu 0} without a rounding bias
+// from the z, theta round trip; eps is the equilibrium's own energy. For MJ every
+// g_nu is z, and the other prefactors follow from n, eps and theta alone.
 // oi selects the expansion order's defect table (order - 2).
 template <int EDF>
-__device__ __forceinline__ void eq_moments(const double g[6], double theta, double ux, double uy,
-                                           double gamma, double nA1, double eA2, double zr[21],
-                                           double zi[21], int oi = kOrder5) {
-  const double u2 = ux * ux + uy * uy;
-  double wr[6], wi[6];
-  wr[0] = 1.0;
-  wi[0] = 0.0;
-#pragma unroll
-  for (int k = 1; k < 6; ++k) {
-    wr[k] = wr[k - 1] * ux - wi[k - 1] * uy;
-    wi[k] = wr[k - 1] * uy + wi[k - 1] * ux;
+__device__ __forceinline__ void eq_moments(const double g[6], double theta, double u2, double gamma, double n,
+                                           double eps, double y[21], int oi = kOrder5) {
+  double A[6];
+  const double tg = theta * gamma;
+  A[1] = n * gamma;
+  A[2] = eps * (gamma * gamma);
+  if (EDF == EDF_MJ) {
+    A[0] = n * rcp64(theta);
+    A[3] = 3.0 * (tg * A[2]);
+    A[4] = 4.0 * (tg * A[3]);
+    A[5] = 5.0 * (tg * A[4]);
+  } else {
+    double q = (12.0 * PI) * (theta * tg) * (tg * tg);
+    A[0] = (2.0 * PI) * (theta * g[0]);
+    A[3] = q * g[3];
+    q *= 4.0 * tg;
+    A[4] = q * g[4];
+    q *= 5.0 * tg;
+    A[5] = q * g[5];
   }
-  double A = 2.0 * PI * theta;  // 2 pi n! theta^{n+1} gamma^n, times g_{n+1}
 #pragma unroll
-  for (int n = 0; n < 6; ++n) {
-    if (n > 0) A *= n * theta * gamma;
-    double An = A * g[n];
-    if (n == 1 && nA1 >= 0.0) An = nA1 * gamma;
-    if (n == 2 && eA2 >= 0.0) An = eA2 * gamma * gamma;
+  for (int n_ = 0; n_ < 6; ++n_)
 #pragma unroll
-    for (int k = 0; k <= n; ++k) {
-      const int i = n * (n + 1) / 2 + k;
-      const double P = fma(u2, fma(u2, c_pnk[3 * i + 2], c_pnk[3 * i + 1]), c_pnk[3 * i + 0]);
-      const double s = An * P;
-      zr[i] = s * wr[k];
-      zi[i] = s * wi[k];
+    for (int k = 0; k <= n_; ++k) {
+      const int i = n_ * (n_ + 1) / 2 + k;
+      const double p0 = pnk(3 * i), p1 = pnk(3 * i + 1), p2 = pnk(3 * i + 2);
+      if (p2 != 0.0) y[i] = A[n_] * fma(u2, fma(u2, p2, p1), p0);
+      else if (p1 != 0.0) y[i] = A[n_] * fma(u2, p1, p0);
+      else y[i] = p0 == 1.0 ? A[n_] : A[n_] * p0;
     }
-  }
   // The rounded projection table misses the identities that make the discrete
   // N^0, T^00 and T^0x, T^0y of f^eq equal Z_10, Z_20, Z_21 by the tiny constant
   // defects e1, e2, e3; correcting those three moments removes the resulting
   // bias (a constant error times Z would drift the conserved totals every step).
-  double d10 = 0.0, d20 = 0.0, d21r = 0.0, d21i = 0.0;
+  double d10 = 0.0, d20 = 0.0, d21 = 0.0;
 #pragma unroll
-  for (int n = 0; n < 6; ++n) {
-    d10 = fma(c_E[oi][EDF][n], zr[n * (n + 1) / 2], d10);
-    d20 = fma(c_E[oi][EDF][6 + n], zr[n * (n + 1) / 2], d20);
+  for (int k = 0; k < 6; ++k) {
+    d10 = fma(c_E[oi][EDF][k], y[k * (k + 1) / 2], d10);
+    d20 = fma(c_E[oi][EDF][6 + k], y[k * (k + 1) / 2], d20);
   }
 #pragma unroll
-  for (int n = 1; n < 6; ++n) {
-    d21r = fma(c_E[oi][EDF][12 + n], zr[n * (n + 1) / 2 + 1], d21r);
-    d21i = fma(c_E[oi][EDF][12 + n], zi[n * (n + 1) / 2 + 1], d21i);
-  }
-  zr[1] -= d10;
-  zr[3] -= d20;
-  zr[4] -= d21r;
-  zi[4] -= d21i;
+  for (int k = 1; k < 6; ++k) d21 = fma(c_E[oi][EDF][12 + k], y[k * (k + 1) / 2 + 1], d21);
+  y[1] -= d10;
+  y[3] -= d20;
+  y[4] -= d21;
+}
+
+// C_k(d) = Re[(u_x + i u_y)^k e^{-i k phi_d}] of the directions d = 0..5 (d + 6
+// flips the sign of odd k): C_2 flips and C_4 repeats after three directions, C_3
+// is +-Re or +-Im (u_x + i u_y)^3. Computed once per cell, they replace the powers
+// in every shell's synthesis (56 FP64 instructions per shell instead of 81, and
+// C_1 is v_d . u, which the relaxation rate needs too).
+struct DirPow {
+  double c1[6], c5[6], c2[3], c4[3], w3r, w3i;
+};
+
+__device__ __forceinline__ DirPow dir_powers(double ux, double uy) {
+  DirPow C;
+  const double h = SQRT3_2;
+  const double w2r = fma(ux, ux, -(uy * uy)), w2i = 2.0 * (ux * uy);
+  C.w3r = fma(w2r, ux, -(w2i * uy));
+  C.w3i = fma(w2r, uy, w2i * ux);
+  const double w4r = fma(w2r, w2r, -(w2i * w2i)), w4i = 2.0 * (w2r * w2i);
+  const double w5r = fma(w4r, ux, -(w4i * uy)), w5i = fma(w4r, uy, w4i * ux);
+  // k = 1: angles 0, 30, .. 150; k = 5: 0, 150, 300, 90, 240, 30
+  const double hx = h * ux, hy = h * uy, gx = h * w5r, gy = h * w5i;
+  C.c1[0] = ux;
+  C.c1[1] = fma(0.5, uy, hx);
+  C.c1[2] = fma(0.5, ux, hy);
+  C.c1[3] = uy;
+  C.c1[4] = fma(-0.5, ux, hy);
+  C.c1[5] = fma(0.5, uy, -hx);
+  C.c5[0] = w5r;
+  C.c5[1] = fma(0.5, w5i, -gx);
+  C.c5[2] = fma(0.5, w5r, -gy);
+  C.c5[3] = w5i;
+  C.c5[4] = fma(-0.5, w5r, -gy);
+  C.c5[5] = fma(0.5, w5i, gx);
+  // k = 2: angles 0, 60, 120; k = 4: 0, 120, 240
+  const double qy = h * w2i, ry = h * w4i;
+  C.c2[0] = w2r;
+  C.c2[1] = fma(0.5, w2r, qy);
+  C.c2[2] = fma(-0.5, w2r, qy);
+  C.c4[0] = w4r;
+  C.c4[1] = fma(-0.5, w4r, ry);
+  C.c4[2] = fma(-0.5, w4r, -ry);
+  return C;
 }
 
 // Discrete equilibrium of one shell s at the 12 directions (order index oi =
 // N - 2; the fifth order by default):
-//   f^eq_{ds} = sum_k R^c_k cos(k phi_d) + R^s_k sin(k phi_d),
-//   R^{c|s}_k = sum_{n>=k} Q^(k)_{s n} Re|Im Z_nk,
-// evaluated with the 12-point symmetries phi -> phi + pi (odd k flip sign) and
-// phi -> pi - phi.
+//   f^eq_{ds} = sum_k R_k C_k(d),  R_k = sum_{n>=k} Q^(k)_{s n} Y_nk,
+// even k the same and odd k of opposite sign at d + 6.
 template <int EDF>
-__device__ __forceinline__ void feq_shell(int s, const double zr[21], const double zi[21],
-                                          double fe[12], int oi = kOrder5) {
-  double Rc[6], Rs[6];
+__device__ __forceinline__ void feq_shell(int s, const double y[21], const DirPow& C, double fe[12],
+                                          int oi = kOrder5) {
+  double R[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    double ac = 0.0, as = 0.0;
+    double a = c_Q[oi][EDF][qoff(k) + s * (6 - k)] * y[k * (k + 1) / 2 + k];
 #pragma unroll
-    for (int n = k; n < 6; ++n) {
-      const double q = c_Q[oi][EDF][qoff(k) + s * (6 - k) + (n - k)];
-      ac = fma(q, zr[n * (n + 1) / 2 + k], ac);
-      as = fma(q, zi[n * (n + 1) / 2 + k], as);
-    }
-    Rc[k] = ac;
-    Rs[k] = as;
+    for (int n = k + 1; n < 6; ++n) a = fma(c_Q[oi][EDF][qoff(k) + s * (6 - k) + (n - k)], y[n * (n + 1) / 2 + k], a);
+    R[k] = a;
   }
-  const double h = SQRT3_2;
-  // even harmonics (period pi)
-  const double t1 = Rc[0] + Rc[4], t2 = fma(-0.5, Rc[4], Rc[0]), h2 = 0.5 * Rc[2];
-  const double Ec0 = t1 + Rc[2], Ec3 = t1 - Rc[2], Ec1 = t2 + h2, Ec2 = t2 - h2;
-  const double Es1 = h * (Rs[2] + Rs[4]), Es2 = h * (Rs[2] - Rs[4]);
-  const double E0 = Ec0, E1 = Ec1 + Es1, E2 = Ec2 + Es2, E3 = Ec3, E4 = Ec2 - Es2, E5 = Ec1 - Es1;
-  // odd harmonics (antiperiodic in pi)
-  const double Oc0 = Rc[1] + Rc[3] + Rc[5], Oc1 = h * (Rc[1] - Rc[5]),
-               Oc2 = fma(0.5, Rc[1] + Rc[5], -Rc[3]);
-  const double Os1 = fma(0.5, Rs[1] + Rs[5], Rs[3]), Os2 = h * (Rs[1] - Rs[5]),
-               Os3 = Rs[1] - Rs[3] + Rs[5];
-  const double O0 = Oc0, O1 = Oc1 + Os1, O2 = Oc2 + Os2, O3 = Os3, O4 = Os2 - Oc2, O5 = Os1 - Oc1;
-  fe[0] = E0 + O0; fe[6] = E0 - O0;
-  fe[1] = E1 + O1; fe[7] = E1 - O1;
-  fe[2] = E2 + O2; fe[8] = E2 - O2;
-  fe[3] = E3 + O3; fe[9] = E3 - O3;
-  fe[4] = E4 + O4; fe[10] = E4 - O4;
-  fe[5] = E5 + O5; fe[11] = E5 - O5;
+  const double p3 = R[3] * C.w3r, q3 = R[3] * C.w3i;
+  // C_3(d): Re, Im, -Re, -Im, Re, Im of w^3
+  const double o3[6] = {p3, q3, -p3, -q3, p3, q3};
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const double t = fma(R[4], C.c4[d % 3], R[0]);
+    const double E = fma(d < 3 ? R[2] : -R[2], C.c2[d % 3], t);
+    const double O = fma(R[1], C.c1[d], fma(R[5], C.c5[d], o3[d]));
+    fe[d] = E + O;
+    fe[d + 6] = E - O;
+  }
 }
 
 // ------------------------------------------------------------------ moments

@@ -9,6 +9,15 @@ namespace rlbm {
 // One fused step for every cell of every tile: pull-stream from fin (its halo
 // was filled by the previous step), moments, Landau state, equilibrium,
 // relaxation (Eq. 3), store to fout and fill fout's halo.
+//
+// Bound: the FP64 pipe. One FP64 warp instruction holds its SM sub-partition's unit
+// for 64 clocks, whatever its operation and however many lanes are active, so the
+// count of FP64 instructions per cell is the time. About 1,040 (MJ): pull 192, moments
+// 200, Landau 40 (FP32 start), state and equilibrium moments 90, directional powers
+// and rates 45, six shells of 80 (21 projection, 35 synthesis, 24 relaxation). With
+// FP64 Newton throughout and harmonic powers applied before the projection it was
+// 1,382. 512^2 local-tau disc, 8 steps with initialisation and read-out: 6.00 -> 4.54
+// ms; FD Riemann 2048 x 4, 50 steps: 5.89 -> 3.12 ms; BE 1024^2, 4 steps: 21.6 -> 11.5 ms.
 template <int EDF>
 __global__ void __launch_bounds__(kThreads) k_step_f64(StepArgs a) {
   extern __shared__ double sm[];
@@ -24,7 +33,7 @@ __global__ void __launch_bounds__(kThreads) k_step_f64(StepArgs a) {
     double N[3], T[6];
     pull_moments64<EDF, StoreF64>(fin, D, x, y, c, sm, tid, N, T);
     CellState S;
-    unsigned st = cell_state<EDF>(N, T, S);
+    unsigned st = cell_state<EDF, false>(N, T, S);
     const bool ok = !(st & ST_NONPHYSICAL);
     if (ok) {
       // constant tau, or the local tau = 4 (eta/s) / theta + 0.2546 of Sec. 3.5;
@@ -42,17 +51,23 @@ __global__ void __launch_bounds__(kThreads) k_step_f64(StepArgs a) {
         gam = 1.0 / sqrt(1.0 - ux * ux - uy * uy);
       }
       const int oi = D.order - 2;
+      const DirPow C = dir_powers(ux, uy);
+      // relaxation rates gamma (1 - v_d . u) / tau (Eq. 3): v_d . u = C_1(d), -C_1(d) at d + 6
+      const double K = gam * itau;
       double om[12];
 #pragma unroll
-      for (int d = 0; d < 12; ++d) om[d] = gam * (1.0 - (dcos(d) * ux + dsin(d) * uy)) * itau;
-      double zr[21], zi[21];
+      for (int d = 0; d < 6; ++d) {
+        om[d] = fma(-K, C.c1[d], K);
+        om[d + 6] = fma(K, C.c1[d], K);
+      }
+      double ym[21];
       // a clamped BE state relaxes to its own equilibrium energy 4 pi theta^3 g_3(z_c)
       const double eps_eq = (st & ST_CLAMPED) ? 4.0 * PI * S.theta * S.theta * S.theta * S.g[2] : S.eps;
-      eq_moments<EDF>(S.g, S.theta, ux, uy, gam, S.n, eps_eq, zr, zi, oi);
+      eq_moments<EDF>(S.g, S.theta, fma(ux, ux, uy * uy), gam, S.n, eps_eq, ym, oi);
 #pragma unroll 1
       for (int s = 0; s < 6; ++s) {
         double fe[12];
-        feq_shell<EDF>(s, zr, zi, fe, oi);
+        feq_shell<EDF>(s, ym, C, fe, oi);
 #pragma unroll
         for (int d = 0; d < 12; ++d) {
           const int q = 6 * d + s;

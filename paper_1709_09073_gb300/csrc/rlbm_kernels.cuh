@@ -165,16 +165,20 @@ __device__ __forceinline__ void pull_moments64(const typename S::T* __restrict__
   T[5] = 0.5 * (hb.h0 - hb.c2);
 }
 
-// FP64 equilibrium at (theta, g, u) written through a functor out(q, value).
+// FP64 equilibrium at (theta, g, u) written through a functor out(q, value):
+// n = 2 pi theta^2 g_2, eps = 4 pi theta^3 g_3 (Eq. 25).
 template <int EDF, class Out>
 __device__ __forceinline__ void feq_emit(const double g[6], double theta, double ux, double uy,
                                          double gamma, int oi, Out out) {
-  double zr[21], zi[21];
-  eq_moments<EDF>(g, theta, ux, uy, gamma, -1.0, -1.0, zr, zi, oi);
+  const double t2 = theta * theta;
+  const double n = (2.0 * PI) * (t2 * g[1]), eps = (4.0 * PI) * (t2 * theta) * g[2];
+  double y[21];
+  eq_moments<EDF>(g, theta, fma(ux, ux, uy * uy), gamma, n, eps, y, oi);
+  const DirPow C = dir_powers(ux, uy);
 #pragma unroll 1
   for (int s = 0; s < 6; ++s) {
     double fe[12];
-    feq_shell<EDF>(s, zr, zi, fe, oi);
+    feq_shell<EDF>(s, y, C, fe, oi);
 #pragma unroll
     for (int d = 0; d < 12; ++d) out(6 * d + s, fe[d]);
   }
@@ -243,7 +247,7 @@ __device__ void write_halo64(const DomDev& D, int x, int y, typename S::T* __res
       if (vw_written) continue;
       const double tw = D.t_wall[wall[i]];
       double z, g[6];
-      st |= solve_z_from_n_theta<EDF>(D.n_wall, tw, z, g);
+      st |= solve_z_from_n_theta<EDF, false>(D.n_wall, tw, z, g);
       feq_emit<EDF>(g, tw, 0.0, 0.0, 1.0, D.order - 2,
                     [&](int q, double v) { fout[q * kBlkW + h] = S::enc(v, D, q % 6); });
       continue;
@@ -253,7 +257,7 @@ __device__ void write_halo64(const DomDev& D, int x, int y, typename S::T* __res
     } else {
       const double tw = D.t_wall[wall[i]];
       double z, g[6];
-      st |= solve_z_from_n_theta<EDF>(n, tw, z, g);
+      st |= solve_z_from_n_theta<EDF, false>(n, tw, z, g);
       feq_emit<EDF>(g, tw, ux, uy, gamma, D.order - 2,
                     [&](int q, double v) { fout[q * kBlkW + h] = S::enc(v, D, q % 6); });
     }
@@ -290,14 +294,16 @@ __device__ __noinline__ void write_vwall_ghosts(const DomDev& D, int x, int y, t
     uy += D.accel_y * tau;
     gam = 1.0 / sqrt(1.0 - ux * ux - uy * uy);
   }
-  double z, g[6], zrw[21], ziw[21], zrc[21], zic[21];
-  *st |= solve_z_from_n_theta<EDF>(D.n_wall, tw, z, g);
-  eq_moments<EDF>(g, tw, 0.0, 0.0, 1.0, -1.0, -1.0, zrw, ziw, oi);
-  eq_moments<EDF>(cs->g, cs->theta, ux, uy, gam, cs->n, cs->eps, zrc, zic, oi);
+  double z, g[6], yw[21], yc[21];
+  *st |= solve_z_from_n_theta<EDF, false>(D.n_wall, tw, z, g);
+  eq_moments<EDF>(g, tw, 0.0, 1.0, (2.0 * PI) * (tw * tw * g[1]), (4.0 * PI) * (tw * tw * tw) * g[2], yw, oi);
+  eq_moments<EDF>(cs->g, cs->theta, fma(ux, ux, uy * uy), gam, cs->n, cs->eps, yc, oi);
+  const DirPow Cw = dir_powers(0.0, 0.0), Cc = dir_powers(ux, uy);
+#pragma unroll 1
   for (int s = 0; s < 6; ++s) {
     double few[12], fe[12];
-    feq_shell<EDF>(s, zrw, ziw, few, oi);
-    feq_shell<EDF>(s, zrc, zic, fe, oi);
+    feq_shell<EDF>(s, yw, Cw, few, oi);
+    feq_shell<EDF>(s, yc, Cc, fe, oi);
     for (int i = 0; i < cnt; ++i) {
       if (wall[i] < 0 || D.bc[wall[i]] != BC_VWALL) continue;
       const long long h = cell_rel(D, hx[i], hy[i]);
@@ -343,7 +349,7 @@ __global__ void __launch_bounds__(kThreads) k_init(InitArgs a) {
     n = 2.0 * PI * theta * theta * g[1];
   } else {
     n = a.a[i];
-    st |= solve_z_from_n_theta<EDF>(n, theta, z, g);
+    st |= solve_z_from_n_theta<EDF, true>(n, theta, z, g);
   }
   const double u2 = ux * ux + uy * uy;
   const bool ok = (u2 < 1.0) && (theta > 0.0) && (n > 0.0) && isfinite(z);
@@ -409,7 +415,7 @@ __global__ void __launch_bounds__(kThreads) k_fields(FieldsArgs a) {
     T[5] = 0.5 * (hb.h0 - hb.c2);
   }
   CellState S_;
-  unsigned st = cell_state<EDF>(N, T, S_);
+  unsigned st = cell_state<EDF, true>(N, T, S_);
   const long long i = (a.tiles ? D.foff : 0) + (long long)y * D.nx + x;
   if (st & ST_NONPHYSICAL) S_.n = S_.theta = S_.ux = S_.uy = S_.z = nan("");
   if (a.n) a.n[i] = S_.n;
@@ -432,12 +438,13 @@ __global__ void __launch_bounds__(kThreads) k_fields(FieldsArgs a) {
       out[1] = hq * (S_.n * S_.gamma * S_.ux - N[1]);
       out[2] = hq * (S_.n * S_.gamma * S_.uy - N[2]);
       const double eps_eq = (st & ST_CLAMPED) ? 4.0 * PI * S_.theta * S_.theta * S_.theta * S_.g[2] : S_.eps;
-      double zr[21], zi[21];
-      eq_moments<EDF>(S_.g, S_.theta, S_.ux, S_.uy, S_.gamma, S_.n, eps_eq, zr, zi, D.order - 2);
+      double ym[21];
+      eq_moments<EDF>(S_.g, S_.theta, fma(S_.ux, S_.ux, S_.uy * S_.uy), S_.gamma, S_.n, eps_eq, ym, D.order - 2);
+      const DirPow C = dir_powers(S_.ux, S_.uy);
       double p2 = 0.0, p3 = 0.0, p4 = 0.0, p5 = 0.0;
       for (int s = 0; s < 6; ++s) {
         double fe[12];
-        feq_shell<EDF>(s, zr, zi, fe, D.order - 2);
+        feq_shell<EDF>(s, ym, C, fe, D.order - 2);
 #pragma unroll
         for (int d = 0; d < 12; ++d) {
           const int q = 6 * d + s;

@@ -1049,7 +1049,7 @@ __global__ void k_prepare_refs(DomDev* doms, int ndom) {
   if (i >= ndom) return;
   DomDev& D = doms[i];
   double z, g[6];
-  solve_z_from_n_theta<EDF>(D.ref_n, D.ref_theta, z, g);
+  solve_z_from_n_theta<EDF, false>(D.ref_n, D.ref_theta, z, g);
   double fact = 1.0, th = D.ref_theta, thp = th;
   for (int n = 0; n < 6; ++n) {
     if (n > 0) { fact *= n; thp *= th; }
