@@ -239,9 +239,9 @@ cudaError_t capture(rlbm_ctx* h, int from, int nsteps, cudaGraphExec_t* out) {
 }
 
 // TMA descriptors of the staged mixed step, written into `out` as
-// [copy][domain]: a 4D tensor {32 lanes, 72 planes, nblk blocks, ny + 2 rows}
-// of the copy's elements (the halo ring included), boxes {32, 6, 3, kTileH + 2} (one
-// direction's six shell planes, the tile's block and its neighbours, rows
+// [copy][domain]: a 4D tensor {64 elements, 36 plane pairs, nblk blocks, ny + 2 rows}
+// of the copy's elements (the halo ring included), boxes {64, 3, 3, kTileH + 2} (one
+// direction's three plane pairs, the tile's block and its neighbours, rows
 // y0-1 .. y0+kTileH), zero fill outside. Returns false if the driver offers no
 // encoder or refuses a descriptor; the handle then has only the L1 variant.
 bool encode_tmaps(const rlbm_ctx* h, std::vector<unsigned char>& out) {
@@ -265,9 +265,9 @@ bool encode_tmaps(const rlbm_ctx* h, std::vector<unsigned char>& out) {
     for (size_t i = 0; i < nd; ++i) {
       const DomDev& D = h->L.dd[i];
       char* base = static_cast<char*>(h->pop[copy]) + (size_t)D.off * es;  // 256-byte aligned
-      const cuuint64_t dims[4] = {(cuuint64_t)kBlkW, (cuuint64_t)kNq, (cuuint64_t)D.nblk, (cuuint64_t)D.ny + 2};
-      const cuuint64_t strides[3] = {(cuuint64_t)kBlkW * es, (cuuint64_t)kBlk * es, (cuuint64_t)D.pitch * es};
-      const cuuint32_t box[4] = {(cuuint32_t)kBlkW, (cuuint32_t)kBoxPlanes, (cuuint32_t)kBoxBlocks,
+      const cuuint64_t dims[4] = {(cuuint64_t)kSegW, (cuuint64_t)kPairs, (cuuint64_t)D.nblk, (cuuint64_t)D.ny + 2};
+      const cuuint64_t strides[3] = {(cuuint64_t)kSegW * es, (cuuint64_t)kBlk * es, (cuuint64_t)D.pitch * es};
+      const cuuint32_t box[4] = {(cuuint32_t)kSegW, (cuuint32_t)kBoxPairs, (cuuint32_t)kBoxBlocks,
                                  (cuuint32_t)kBoxRows};
       CUtensorMap* m = reinterpret_cast<CUtensorMap*>(out.data() + ((size_t)copy * nd + i) * kTensorMapBytes);
       if (encode(m, dt, 4, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -304,10 +304,11 @@ struct RowArgs {
 };
 
 // Raw element copy between a packed [30][nx + 2] face and one row of 30
-// planes, both faces in one launch (the storage encoding is kept as is).
+// planes, both faces in one launch, a plane pair per thread (the storage encoding is
+// kept as is; the faces' planes begin at even ones).
 template <class T>
 __global__ void k_rows(RowArgs a) {
-  const long long w = a.D.nx + 2, per = kSlabPlanes * w;
+  const long long w = a.D.nx + 2, per = kSlabPlanes / 2 * w;
   T* pop = static_cast<T*>(a.pop);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < 2 * per;
        e += (long long)gridDim.x * blockDim.x) {
@@ -320,18 +321,24 @@ __global__ void k_rows(RowArgs a) {
     const int q0 = (side == 0) == (a.unpack != 0) ? kPlanesUp : kPlanesDown;
     const int y = a.unpack ? (side ? a.D.ny : -1) : (side ? a.D.ny - 1 : 0);
     int x = (int)xx - 1;
-    // a sent row's periodic x ghosts are its wrapped end cells (the L1 step
-    // leaves the images unwritten)
+    // a sent row's periodic x ghosts are its wrapped end cells (the steps leave the
+    // images unwritten)
     if (!a.unpack && a.D.bc[0] == BC_PERIODIC) x = x < 0 ? a.D.nx - 1 : (x == a.D.nx ? 0 : x);
-    const long long idx = cell_pos(a.D, x, y) + (q0 + k) * kBlkW;
-    if (a.unpack) pop[idx] = buf[r];
-    else buf[r] = pop[idx];
+    Pair<T>* cell = reinterpret_cast<Pair<T>*>(pop + cell_pos(a.D, x, y) + plane_off(q0 + 2 * (int)k));
+    T* f = buf + 2 * k * w + xx;
+    if (a.unpack) {
+      *cell = Pair<T>{f[0], f[w]};
+    } else {
+      const Pair<T> v = *cell;
+      f[0] = v.x;
+      f[w] = v.y;
+    }
   }
 }
 
 // Periodic halo images of every domain of a population copy, copied from the
-// interior cells they map to (raw elements, all 72 planes): pass 0 the x
-// images of rows -1..ny, then pass 1 the y images of columns -1..nx (so the
+// interior cells they map to (raw elements, all 72 planes, a pair per thread): pass 0
+// the x images of rows -1..ny, then pass 1 the y images of columns -1..nx (so the
 // corners take the images of the x ghosts). The result is the halo the
 // producing step would have written with its images on.
 template <class T>
@@ -340,12 +347,12 @@ __global__ void k_images(const DomDev* doms, int ndom, void* pop_, int pass) {
   for (int dm = blockIdx.y; dm < ndom; dm += gridDim.y) {
     const DomDev& D = doms[dm];
     if (D.bc[pass == 0 ? 0 : 2] != BC_PERIODIC) continue;
-    const long long len = pass == 0 ? D.ny + 2 : D.nx + 2, per = 72 * len;
+    const long long len = pass == 0 ? D.ny + 2 : D.nx + 2, per = kPairs * len;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < 2 * per;
          e += (long long)gridDim.x * blockDim.x) {
       const int side = e >= per;
       const long long r = e - side * per;
-      const int q = (int)(r / len), k = (int)(r % len) - 1;
+      const int q = 2 * (int)(r / len), k = (int)(r % len) - 1;
       long long dst, src;
       if (pass == 0) {
         dst = cell_pos(D, side ? D.nx : -1, k);
@@ -354,7 +361,8 @@ __global__ void k_images(const DomDev* doms, int ndom, void* pop_, int pass) {
         dst = cell_pos(D, k, side ? D.ny : -1);
         src = cell_pos(D, k, side ? 0 : D.ny - 1);
       }
-      pop[dst + q * kBlkW] = pop[src + q * kBlkW];
+      *reinterpret_cast<Pair<T>*>(pop + dst + plane_off(q)) =
+          *reinterpret_cast<const Pair<T>*>(pop + src + plane_off(q));
     }
   }
 }
@@ -388,8 +396,8 @@ int slab_rows(rlbm_handle h, int domain, void* lo, void* hi, int unpack) {
   a.pop = h->pop[h->cur];
   a.face[0] = lo;
   a.face[1] = hi;
-  const long long n = 2LL * kSlabPlanes * (D.nx + 2);
-  // one element per thread, at most 8 blocks of 256 per SM (152 SMs); the loop strides beyond
+  const long long n = 1LL * kSlabPlanes * (D.nx + 2);
+  // one plane pair per thread, at most 8 blocks of 256 per SM (152 SMs); the loop strides beyond
   const int grid = (int)std::min<long long>((n + 255) / 256, 8 * 152);
   switch (es) {
     case 8: k_rows<unsigned long long><<<grid, 256, 0, h->stream>>>(a); break;

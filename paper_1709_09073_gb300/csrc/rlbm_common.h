@@ -22,16 +22,30 @@ constexpr double ZC = 1.0 - 1.0e-7;  // BE reference fugacity, Eq. (15)
 constexpr double SQRT3_2 = 0.86602540378443864676372317075294;
 
 // Population layout: blocks of 32 cells of a row, each block holding all 72
-// populations of its cells ("array of structures of arrays"): element (q, x, y),
-// x in [-1, nx], y in [-1, ny] (the halo ring included), lives at
-//   off + (y + 1) * pitch + ((x + 32) / 32) * kBlk + q * kBlkW + (x + 32) % 32,
-// so a warp's access to one population of 32 cells is one aligned 32-element
-// segment, the 72 segments of a block are contiguous, and the offset of plane
-// q is the constant q * kBlkW. Block 0 of a row holds x = -32 .. -1 (only x = -1
-// is used); pitch = nblk * kBlk with nblk = (nx + 32) / 32 + 1 blocks per row.
+// populations of its cells, neighbouring planes in pairs per cell: element
+// (q, x, y), x in [-1, nx], y in [-1, ny] (the halo ring included), lives at
+//   off + (y + 1) * pitch + ((x + 32) / 32) * kBlk + plane_off(q) + 2 * ((x + 32) % 32),
+// so a warp reads or writes the two planes of a pair (shells s, s + 1 of one
+// direction) of 32 cells as one aligned 64-element segment with one instruction a
+// lane (8 bytes in FP32, 4 in the 16-bit storages, 16 in FP64), the 36 segments of a
+// block are contiguous, and the offset of plane q is a constant. Block 0 of a row
+// holds x = -32 .. -1 (only x = -1 is used); pitch = nblk * kBlk with
+// nblk = (nx + 32) / 32 + 1 blocks per row. With one plane per segment the mixed
+// step issued twice the loads and stores (see k_step_mixed).
 constexpr int kBlkW = 32;           // cells per x block
 constexpr int kNq = 72;             // populations per cell
 constexpr int kBlk = kNq * kBlkW;   // elements per x block
+constexpr int kPairs = kNq / 2;     // plane pairs per cell
+constexpr int kSegW = 2 * kBlkW;    // elements of a pair's segment in a block
+
+// Offset of plane q from a cell's first element; the planes 2k and 2k + 1 are adjacent.
+__host__ __device__ constexpr int plane_off(int q) { return (q >> 1) * kSegW + (q & 1); }
+
+// A pair of elements, loaded and stored as one.
+template <class T>
+struct alignas(2 * sizeof(T)) Pair {
+  T x, y;
+};
 
 struct DomDev {
   int nx, ny, nblk, pad0;
@@ -113,11 +127,11 @@ struct StepArgs {
 
 constexpr unsigned long long kDefaultWaitNs = 1000000000ull;  // one second
 
-// Element index of cell (x, y), plane 0 (add q * kBlkW for plane q), from the
+// Element index of cell (x, y), plane 0 (add plane_off(q) for plane q), from the
 // start of the domain (cell_rel) or of the population copy (cell_pos).
 __host__ __device__ inline long long cell_rel(const DomDev& D, int x, int y) {
   const int X = x + kBlkW;  // >= 31
-  return (long long)(y + 1) * D.pitch + (long long)(X / kBlkW) * kBlk + (X % kBlkW);
+  return (long long)(y + 1) * D.pitch + (long long)(X / kBlkW) * kBlk + 2 * (X % kBlkW);
 }
 __host__ __device__ inline long long cell_pos(const DomDev& D, int x, int y) { return D.off + cell_rel(D, x, y); }
 
@@ -126,11 +140,11 @@ __host__ __device__ constexpr int blocks_per_row(int nx) { return (nx + kBlkW) /
 
 constexpr int kTensorMapBytes = 128;  // sizeof(CUtensorMap), 64-byte aligned in memory
 
-// TMA box of the staged mixed step: for one direction, the six shell planes of
+// TMA box of the staged mixed step: for one direction, the three plane pairs of
 // the tile's x block and its two neighbours over rows y0-1 .. y0+kTileH, i.e. a
-// box {32 lanes, 6 planes, 3 blocks, kTileH + 2 rows} of the 4D tensor
-// {32 lanes, 72 planes, nblk blocks, ny + 2 rows}.
-constexpr int kBoxRows = kTileH + 2, kBoxBlocks = 3, kBoxPlanes = 6;
-constexpr int kBoxElems = kBlkW * kBoxPlanes * kBoxBlocks * kBoxRows;
+// box {64 elements, 3 pairs, 3 blocks, kTileH + 2 rows} of the 4D tensor
+// {64 elements, 36 pairs, nblk blocks, ny + 2 rows}.
+constexpr int kBoxRows = kTileH + 2, kBoxBlocks = 3, kBoxPairs = 3;
+constexpr int kBoxElems = kSegW * kBoxPairs * kBoxBlocks * kBoxRows;
 
 }  // namespace rlbm

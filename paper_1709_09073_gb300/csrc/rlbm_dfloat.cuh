@@ -7,67 +7,90 @@
 // round-to-nearest intrinsics, which the compiler neither reassociates nor
 // contracts into an FMA with a neighbouring product: the error-free
 // transformations are exact only as written, and every kernel that inlines
-// them gets the same roundings.
+// them gets the same roundings. Each is written once for scalars and for pairs (f2):
+// df2 holds two double-floats, the x and y components of a vector, at the
+// instruction count of one.
 #pragma once
 #include <cuda_runtime.h>
 
+#include "rlbm_f32x2.cuh"
+
 namespace rlbm {
 
-struct df {
-  float hi, lo;
+template <class V>
+struct dft {
+  V hi, lo;
 };
+using df = dft<float>;
+using df2 = dft<f2>;
 
-__device__ __forceinline__ df df_make(float hi, float lo) {
-  df r;
+template <class V>
+__device__ __forceinline__ dft<V> df_make(V hi, V lo) {
+  dft<V> r;
   r.hi = hi;
   r.lo = lo;
   return r;
 }
 
+// two double-floats as a pair, and the parts of a pair
+__device__ __forceinline__ df2 df_join(df a, df b) { return df_make(f2_make(a.hi, b.hi), f2_make(a.lo, b.lo)); }
+__device__ __forceinline__ df df_first(df2 a) { return df_make(f2_lo(a.hi), f2_lo(a.lo)); }
+__device__ __forceinline__ df df_second(df2 a) { return df_make(f2_hi(a.hi), f2_hi(a.lo)); }
+__device__ __forceinline__ df2 df_dup(df a) { return df_make(f2_dup(a.hi), f2_dup(a.lo)); }
+
 // s + e = a + b exactly
-__device__ __forceinline__ df two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  const float v = __fsub_rn(s, a);
-  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+template <class V>
+__device__ __forceinline__ dft<V> two_sum(V a, V b) {
+  const V s = vadd(a, b);
+  const V v = vsub(s, a);
+  const V e = vadd(vsub(a, vsub(s, v)), vsub(b, v));
   return df_make(s, e);
 }
 
 // s + e = a + b exactly, requires |a| >= |b|
-__device__ __forceinline__ df quick_two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  return df_make(s, __fsub_rn(b, __fsub_rn(s, a)));
+template <class V>
+__device__ __forceinline__ dft<V> quick_two_sum(V a, V b) {
+  const V s = vadd(a, b);
+  return df_make(s, vsub(b, vsub(s, a)));
 }
 
 // p + e = a * b exactly
-__device__ __forceinline__ df two_prod(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return df_make(p, fmaf(a, b, -p));
+template <class V>
+__device__ __forceinline__ dft<V> two_prod(V a, V b) {
+  const V p = vmul(a, b);
+  return df_make(p, vfma(a, b, vneg(p)));
 }
 
-__device__ __forceinline__ df df_add(df a, df b) {
-  df s = two_sum(a.hi, b.hi);
-  s.lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
+template <class V>
+__device__ __forceinline__ dft<V> df_add(dft<V> a, dft<V> b) {
+  dft<V> s = two_sum(a.hi, b.hi);
+  s.lo = vadd(s.lo, vadd(a.lo, b.lo));
   return quick_two_sum(s.hi, s.lo);
 }
 
-__device__ __forceinline__ df df_add(df a, float b) {
-  df s = two_sum(a.hi, b);
-  s.lo = __fadd_rn(s.lo, a.lo);
+template <class V>
+__device__ __forceinline__ dft<V> df_add(dft<V> a, V b) {
+  dft<V> s = two_sum(a.hi, b);
+  s.lo = vadd(s.lo, a.lo);
   return quick_two_sum(s.hi, s.lo);
 }
 
-__device__ __forceinline__ df df_neg(df a) { return df_make(-a.hi, -a.lo); }
-__device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df_neg(b)); }
+template <class V>
+__device__ __forceinline__ dft<V> df_neg(dft<V> a) { return df_make(vneg(a.hi), vneg(a.lo)); }
+template <class V>
+__device__ __forceinline__ dft<V> df_sub(dft<V> a, dft<V> b) { return df_add(a, df_neg(b)); }
 
-__device__ __forceinline__ df df_mul(df a, df b) {
-  df p = two_prod(a.hi, b.hi);
-  p.lo = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, p.lo));
+template <class V>
+__device__ __forceinline__ dft<V> df_mul(dft<V> a, dft<V> b) {
+  dft<V> p = two_prod(a.hi, b.hi);
+  p.lo = vfma(a.hi, b.lo, vfma(a.lo, b.hi, p.lo));
   return quick_two_sum(p.hi, p.lo);
 }
 
-__device__ __forceinline__ df df_mul(df a, float b) {
-  df p = two_prod(a.hi, b);
-  p.lo = fmaf(a.lo, b, p.lo);
+template <class V>
+__device__ __forceinline__ dft<V> df_mul(dft<V> a, V b) {
+  dft<V> p = two_prod(a.hi, b);
+  p.lo = vfma(a.lo, b, p.lo);
   return quick_two_sum(p.hi, p.lo);
 }
 
@@ -83,14 +106,7 @@ __device__ __forceinline__ df df_rsqrt(df a) {
   return quick_two_sum(g, __fmul_rn(__fmul_rn(0.5f, g), e));
 }
 
-// a / b: FP32 quotient refined once with the double-float remainder
-__device__ __forceinline__ df df_div(df a, df b) {
-  const float q1 = __fdiv_rn(a.hi, b.hi);
-  const df r = df_sub(a, df_mul(b, q1));
-  const float q2 = __fdiv_rn(r.hi, b.hi);
-  return quick_two_sum(q1, q2);
-}
-
-__device__ __forceinline__ float df_to_float(df a) { return __fadd_rn(a.hi, a.lo); }
+template <class V>
+__device__ __forceinline__ V df_to_float(dft<V> a) { return vadd(a.hi, a.lo); }
 
 }  // namespace rlbm

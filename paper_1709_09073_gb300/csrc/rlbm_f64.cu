@@ -74,13 +74,15 @@ __global__ void __launch_bounds__(kThreads) k_step_f64(StepArgs a) {
           const double v = sm[q * kThreads + tid];
           const double r = fma(om[d], fe[d] - v, v);
           sm[q * kThreads + tid] = r;
-          fout[q * kBlkW + c] = r;
         }
       }
       if (touches_vwall(D, x, y)) write_vwall_ghosts<EDF, StoreF64>(D, x, y, fout, sm, tid, &S, &st);
-    } else {
-      for (int q = 0; q < 72; ++q) fout[q * kBlkW + c] = sm[q * kThreads + tid];
     }
+    // f* (or the unrelaxed populations of a non-physical cell), a plane pair per store
+#pragma unroll 4
+    for (int q = 0; q < 72; q += 2)
+      *reinterpret_cast<Pair<double>*>(fout + plane_off(q) + c) =
+          Pair<double>{sm[q * kThreads + tid], sm[(q + 1) * kThreads + tid]};
     write_halo64<EDF, StoreF64>(D, x, y, fout, sm, tid, ok, S.n, S.ux, S.uy, S.gamma, st, ok);
     if (st) atomicOr(a.status, st);
   }

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "rlbm_device.cuh"
+#include "rlbm_f32x2.cuh"
 #include "rlbm_launch.h"
 
 namespace rlbm {
@@ -24,9 +25,11 @@ __host__ __device__ constexpr double dsin(int d) { return dcos((d + 9) % 12); }
 __host__ __device__ constexpr double dabs(double v) { return v < 0.0 ? -v : v; }
 
 // ------------------------------------------------------------ storage policies
-// dec/enc convert between a stored value and the population f in FP64;
-// decf/encf between a stored (or interpolated) value and the FP32 deviation
-// f - fref used by the mixed-precision step.
+// dec/enc convert between a stored value and the population f in FP64. The mixed
+// step works on pairs (shells s, s + 1) in "work units", in which storing is a
+// rounding alone: the FP32 deviation f - fref, divided by the per-shell scale a_s in
+// the 16-bit storages (kScaled). raw2: the stored pair in FP32; work2: in work
+// units; enc2: work units to stored.
 struct StoreF64 {
   using T = double;
   static constexpr int kind = ST_F64;
@@ -37,46 +40,65 @@ struct StoreF64 {
 struct StoreF32 {
   using T = float;
   static constexpr int kind = ST_F32;
+  static constexpr bool kScaled = false;
   __device__ static float raw(T v) { return v; }
   __device__ static double dec(double r, const DomDev&, int) { return r; }
   __device__ static T enc(double f, const DomDev&, int) { return (float)f; }
-  __device__ static float decf(float r, const DomDev& D, int s) { return r - D.fref[s]; }
-  __device__ static T encf(float df, const DomDev& D, int s) { return D.fref[s] + df; }
+  __device__ static f2 raw2(Pair<T> v) { return f2_make(v.x, v.y); }
+  __device__ static f2 work2(f2 r, const DomDev& D, int s) { return vsub(r, f2_make(D.fref[s], D.fref[s + 1])); }
+  __device__ static Pair<T> enc2(f2 w, const DomDev& D, int s) {
+    const f2 r = vadd(f2_make(D.fref[s], D.fref[s + 1]), w);
+    return Pair<T>{f2_lo(r), f2_hi(r)};
+  }
 };
 struct StoreBF16 {
   using T = __nv_bfloat16;
   static constexpr int kind = ST_BF16DEV;
+  static constexpr bool kScaled = true;
   __device__ static float raw(T v) { return __bfloat162float(v); }
   __device__ static double dec(double h, const DomDev& D, int s) { return (double)D.fref[s] + (double)D.a_s[s] * h; }
   __device__ static T enc(double f, const DomDev& D, int s) {
     return __float2bfloat16_rn((float)((f - (double)D.fref[s]) * (double)D.b_s[s]));
   }
-  __device__ static float decf(float h, const DomDev& D, int s) { return D.a_s[s] * h; }
-  __device__ static T encf(float df, const DomDev& D, int s) { return __float2bfloat16_rn(df * D.b_s[s]); }
+  __device__ static f2 raw2(Pair<T> v) {  // a BF16 is the upper half of an FP32
+    const unsigned w = *reinterpret_cast<const unsigned*>(&v);
+    return f2_make(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+  }
+  __device__ static f2 work2(f2 r, const DomDev&, int) { return r; }
+  __device__ static Pair<T> enc2(f2 w, const DomDev&, int) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(f2_lo(w), f2_hi(w));
+    return Pair<T>{h.x, h.y};
+  }
 };
 struct StoreF16 {
   using T = __half;
   static constexpr int kind = ST_F16DEV;
+  static constexpr bool kScaled = true;
   __device__ static float raw(T v) { return __half2float(v); }
   __device__ static double dec(double h, const DomDev& D, int s) { return (double)D.fref[s] + (double)D.a_s[s] * h; }
   __device__ static T enc(double f, const DomDev& D, int s) {
     return __float2half_rn((float)((f - (double)D.fref[s]) * (double)D.b_s[s]));
   }
-  __device__ static float decf(float h, const DomDev& D, int s) { return D.a_s[s] * h; }
-  __device__ static T encf(float df, const DomDev& D, int s) { return __float2half_rn(df * D.b_s[s]); }
+  __device__ static f2 raw2(Pair<T> v) { return f2_make(__half2float(v.x), __half2float(v.y)); }
+  __device__ static f2 work2(f2 r, const DomDev&, int) { return r; }
+  __device__ static Pair<T> enc2(f2 w, const DomDev&, int) {
+    const __half2 h = __floats2half2_rn(f2_lo(w), f2_hi(w));
+    return Pair<T>{__low2half(h), __high2half(h)};
+  }
 };
 
 // FP32 absolute deviation h = f - fref: FP32's exponent range covers every
-// shell, so no per-shell scale is needed and decoding/encoding in the mixed
-// step are exact identities.
+// shell, so no per-shell scale is needed and the stored values are the work units.
 struct StoreF32Dev {
   using T = float;
   static constexpr int kind = ST_F32DEV;
+  static constexpr bool kScaled = false;
   __device__ static float raw(T v) { return v; }
   __device__ static double dec(double h, const DomDev& D, int s) { return (double)D.fref[s] + h; }
   __device__ static T enc(double f, const DomDev& D, int s) { return (float)(f - (double)D.fref[s]); }
-  __device__ static float decf(float h, const DomDev&, int) { return h; }
-  __device__ static T encf(float df, const DomDev&, int) { return df; }
+  __device__ static f2 raw2(Pair<T> v) { return f2_make(v.x, v.y); }
+  __device__ static f2 work2(f2 r, const DomDev&, int) { return r; }
+  __device__ static Pair<T> enc2(f2 w, const DomDev&, int) { return Pair<T>{f2_lo(w), f2_hi(w)}; }
 };
 
 // Element offsets, from a cell's own element, of its neighbours x - 1 and
@@ -93,8 +115,8 @@ struct Nbr {
 __device__ __forceinline__ Nbr neighbours(const DomDev& D, int x, int y) {
   const int lane = (x + kBlkW) % kBlkW;
   Nbr n;
-  n.xm = lane ? -1 : -kBlk + (kBlkW - 1);
-  n.xp = lane != kBlkW - 1 ? 1 : kBlk - (kBlkW - 1);
+  n.xm = lane ? -2 : -kBlk + 2 * (kBlkW - 1);
+  n.xp = lane != kBlkW - 1 ? 2 : kBlk - 2 * (kBlkW - 1);
   if (D.bc[0] == BC_PERIODIC) {
     const int span = (int)(cell_rel(D, D.nx - 1, 0) - cell_rel(D, 0, 0));
     if (x == 0) n.xm = span;
@@ -110,27 +132,49 @@ __device__ __forceinline__ Nbr neighbours(const DomDev& D, int x, int y) {
   return n;
 }
 
-// Bilinear interpolated pull of direction d from one plane (Eqs. 17-18): the
+// Bilinear interpolated pull of direction d from one plane pair (Eqs. 17-18): the
 // four grid points around x - v_d with weights |v_x||v_y|, (1-|v_x|)|v_y|,
 // |v_x|(1-|v_y|), (1-|v_x|)(1-|v_y|); axis directions shift by one cell.
-// `pl` points at the cell's own element of the plane. Interpolates the stored
-// values (decoding is affine per plane).
-template <int d, class R, class S>
-__device__ __forceinline__ R pull_one(const typename S::T* __restrict__ pl, const Nbr& nb) {
+// `pl` points at the cell's own element of the pair's first plane. Interpolates the
+// stored values (decoding is affine per plane). R: f2 (the mixed forms) or Pair<double>.
+struct PullF32 {  // FP32 pairs
+  using R = f2;
+  template <class S>
+  __device__ static R raw(Pair<typename S::T> v) { return S::raw2(v); }
+  __device__ static R mul(float w, R v) { return vmul(f2_dup(w), v); }
+  __device__ static R fma(float w, R v, R a) { return vfma(f2_dup(w), v, a); }
+  using W = float;
+};
+struct PullF64 {  // FP64 pairs
+  using R = Pair<double>;
+  template <class S>
+  __device__ static R raw(Pair<typename S::T> v) { return R{(double)S::raw(v.x), (double)S::raw(v.y)}; }
+  __device__ static R mul(double w, R v) { return R{w * v.x, w * v.y}; }
+  __device__ static R fma(double w, R v, R a) { return R{::fma(w, v.x, a.x), ::fma(w, v.y, a.y)}; }
+  using W = double;
+};
+
+template <int d, class A, class S>
+__device__ __forceinline__ typename A::R pull_pair(const typename S::T* __restrict__ pl, const Nbr& nb) {
+  using W = typename A::W;
+  using P = Pair<typename S::T>;
   constexpr double cx = dcos(d), cy = dsin(d);
   constexpr int sx = sgnd(cx), sy = sgnd(cy);
   constexpr double ax = dabs(cx), ay = dabs(cy);
   const long long ox = sx > 0 ? nb.xm : (sx < 0 ? nb.xp : 0);  // to x - sx
   const long long oy = sy > 0 ? nb.ym : (sy < 0 ? nb.yp : 0);   // to y - sy
-  if (ax == 0.0 || ay == 0.0) return (R)S::raw(pl[ox + oy]);
+  if (ax == 0.0 || ay == 0.0) return A::template raw<S>(*reinterpret_cast<const P*>(pl + ox + oy));
   // weights from the rounded |v_x|, |v_y| (one of them is 1/2): every product and
-  // 1 - |v| is exact in R, so the four weights sum to exactly 1 and streaming
+  // 1 - |v| is exact in W, so the four weights sum to exactly 1 and streaming
   // conserves the global sums of every plane
-  constexpr R axr = (R)ax, ayr = (R)ay;
-  constexpr R w1 = axr * ayr, w2 = (R(1) - axr) * ayr, w3 = axr * (R(1) - ayr),
-              w4 = (R(1) - axr) * (R(1) - ayr);
-  const R v1 = (R)S::raw(pl[ox + oy]), v2 = (R)S::raw(pl[oy]), v3 = (R)S::raw(pl[ox]), v4 = (R)S::raw(pl[0]);
-  return fma(w1, v1, fma(w2, v2, fma(w3, v3, w4 * v4)));
+  constexpr W axr = (W)ax, ayr = (W)ay;
+  constexpr W w1 = axr * ayr, w2 = (W(1) - axr) * ayr, w3 = axr * (W(1) - ayr),
+              w4 = (W(1) - axr) * (W(1) - ayr);
+  const P v1 = *reinterpret_cast<const P*>(pl + ox + oy), v2 = *reinterpret_cast<const P*>(pl + oy),
+          v3 = *reinterpret_cast<const P*>(pl + ox), v4 = *reinterpret_cast<const P*>(pl);
+  return A::fma(w1, A::template raw<S>(v1),
+                A::fma(w2, A::template raw<S>(v2),
+                       A::fma(w3, A::template raw<S>(v3), A::mul(w4, A::template raw<S>(v4)))));
 }
 
 // Pull all 72 populations (FP64) into the thread's shared-memory column and
@@ -144,11 +188,15 @@ __device__ __forceinline__ void pull_moments64(const typename S::T* __restrict__
 #define RLBM_PULL_DIR(d)                                                          \
   {                                                                               \
     double a_ = 0.0, b_ = 0.0;                                                    \
-    _Pragma("unroll") for (int s = 0; s < 6; ++s) {                               \
-      const double v = S::dec(pull_one<d, double, S>(fin + c + (6 * d + s) * kBlkW, nb), D, s); \
+    _Pragma("unroll") for (int s = 0; s < 6; s += 2) {                            \
+      const Pair<double> r_ = pull_pair<d, PullF64, S>(fin + c + plane_off(6 * d + s), nb); \
+      const double v = S::dec(r_.x, D, s), w = S::dec(r_.y, D, s + 1);            \
       sm[(6 * d + s) * kThreads + tid] = v;                                       \
+      sm[(6 * d + s + 1) * kThreads + tid] = w;                                   \
       a_ = fma(v, c_p[EDF][s], a_);                                               \
       b_ = fma(v, c_p2[EDF][s], b_);                                              \
+      a_ = fma(w, c_p[EDF][s + 1], a_);                                           \
+      b_ = fma(w, c_p2[EDF][s + 1], b_);                                          \
     }                                                                             \
     A[d] = a_;                                                                    \
     B[d] = b_;                                                                    \
@@ -249,17 +297,17 @@ __device__ void write_halo64(const DomDev& D, int x, int y, typename S::T* __res
       double z, g[6];
       st |= solve_z_from_n_theta<EDF, false>(D.n_wall, tw, z, g);
       feq_emit<EDF>(g, tw, 0.0, 0.0, 1.0, D.order - 2,
-                    [&](int q, double v) { fout[q * kBlkW + h] = S::enc(v, D, q % 6); });
+                    [&](int q, double v) { fout[plane_off(q) + h] = S::enc(v, D, q % 6); });
       continue;
     }
     if (wall[i] < 0 || !have_state) {
-      for (int q = 0; q < 72; ++q) fout[q * kBlkW + h] = S::enc(sm[q * kThreads + tid], D, q % 6);
+      for (int q = 0; q < 72; ++q) fout[plane_off(q) + h] = S::enc(sm[q * kThreads + tid], D, q % 6);
     } else {
       const double tw = D.t_wall[wall[i]];
       double z, g[6];
       st |= solve_z_from_n_theta<EDF, false>(n, tw, z, g);
       feq_emit<EDF>(g, tw, ux, uy, gamma, D.order - 2,
-                    [&](int q, double v) { fout[q * kBlkW + h] = S::enc(v, D, q % 6); });
+                    [&](int q, double v) { fout[plane_off(q) + h] = S::enc(v, D, q % 6); });
     }
   }
 }
@@ -309,7 +357,7 @@ __device__ __noinline__ void write_vwall_ghosts(const DomDev& D, int x, int y, t
       const long long h = cell_rel(D, hx[i], hy[i]);
       for (int d = 0; d < 12; ++d) {
         const int q = 6 * d + s;
-        fout[q * kBlkW + h] = S::enc(few[d] + (sm[q * kThreads + tid] - fe[d]), D, s);
+        fout[plane_off(q) + h] = S::enc(few[d] + (sm[q * kThreads + tid] - fe[d]), D, s);
       }
     }
   }
@@ -360,12 +408,12 @@ __global__ void __launch_bounds__(kThreads) k_init(InitArgs a) {
   if (ok) {
     feq_emit<EDF>(g, theta, ux, uy, gamma, D.order - 2, [&](int q, double v) {
       sm[q * kThreads + tid] = v;
-      f[q * kBlkW + c] = S::enc(v, D, q % 6);
+      f[plane_off(q) + c] = S::enc(v, D, q % 6);
     });
   } else {
     for (int q = 0; q < 72; ++q) {
       sm[q * kThreads + tid] = nan("");
-      f[q * kBlkW + c] = S::enc(nan(""), D, q % 6);
+      f[plane_off(q) + c] = S::enc(nan(""), D, q % 6);
     }
   }
   bool vw = false;
@@ -400,7 +448,7 @@ __global__ void __launch_bounds__(kThreads) k_fields(FieldsArgs a) {
     for (int d = 0; d < 12; ++d) {
       double a_ = 0.0, b_ = 0.0;
       for (int s = 0; s < 6; ++s) {
-        const double v = S::dec((double)S::raw(f[(6 * d + s) * kBlkW + c]), D, s);
+        const double v = S::dec((double)S::raw(f[plane_off(6 * d + s) + c]), D, s);
         a_ = fma(v, c_p[EDF][s], a_);
         b_ = fma(v, c_p2[EDF][s], b_);
       }
@@ -448,7 +496,7 @@ __global__ void __launch_bounds__(kThreads) k_fields(FieldsArgs a) {
 #pragma unroll
         for (int d = 0; d < 12; ++d) {
           const int q = 6 * d + s;
-          const double v = a.streamed ? sm[q * kThreads + tid] : S::dec((double)S::raw(f[q * kBlkW + c]), D, s);
+          const double v = a.streamed ? sm[q * kThreads + tid] : S::dec((double)S::raw(f[plane_off(q) + c]), D, s);
           const double px = c_p[EDF][s] * dcos(d), w = (v - fe[d]) * px * px;
           p2 += w;
           p3 += w * px;
@@ -466,18 +514,33 @@ __global__ void __launch_bounds__(kThreads) k_fields(FieldsArgs a) {
   if (st) atomicOr(a.status, st);
 }
 
-// Raw populations (halo included) <-> FP64 [72][ny+2][nx+2].
+// Raw populations (halo included) <-> FP64 [72][ny+2][nx+2], a plane pair per thread
+// (the planes q0 .. q0 + nq - 1 may begin or end inside a pair).
 template <class S>
 __global__ void k_copy(CopyArgs a) {
   const DomDev& D = a.doms[a.dom];
-  const long long w = D.nx + 2, h = D.ny + 2, tot = (long long)a.nq * w * h;
+  using P = Pair<typename S::T>;
+  const int p0 = a.q0 >> 1, np = ((a.q0 + a.nq - 1) >> 1) - p0 + 1;
+  const long long w = D.nx + 2, wh = w * (D.ny + 2), tot = np * wh;
   typename S::T* pop = static_cast<typename S::T*>(a.pop);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
        e += (long long)gridDim.x * blockDim.x) {
-    const long long q = a.q0 + e / (w * h), r = e % (w * h), yy = r / w, xx = r % w;
-    const long long src = cell_pos(D, (int)xx - 1, (int)yy - 1) + q * kBlkW;
-    if (a.to_dense) a.dense[e] = S::dec((double)S::raw(pop[src]), D, (int)(q % 6));
-    else pop[src] = S::enc(a.dense[e], D, (int)(q % 6));
+    const int q = 2 * (p0 + (int)(e / wh));
+    const long long r = e % wh, yy = r / w, xx = r % w;
+    P* src = reinterpret_cast<P*>(pop + cell_pos(D, (int)xx - 1, (int)yy - 1) + plane_off(q));
+    double* dn = a.dense + (q - a.q0) * wh + r;
+    const bool in0 = q >= a.q0, in1 = q + 1 < a.q0 + a.nq;
+    if (a.to_dense) {
+      const P v = *src;
+      if (in0) dn[0] = S::dec((double)S::raw(v.x), D, q % 6);
+      if (in1) dn[wh] = S::dec((double)S::raw(v.y), D, q % 6 + 1);
+    } else if (in0 && in1) {
+      *src = P{S::enc(dn[0], D, q % 6), S::enc(dn[wh], D, q % 6 + 1)};
+    } else if (in0) {
+      src->x = S::enc(dn[0], D, q % 6);
+    } else {
+      src->y = S::enc(dn[wh], D, q % 6 + 1);
+    }
   }
 }
 

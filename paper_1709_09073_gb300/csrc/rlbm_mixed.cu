@@ -16,10 +16,9 @@ const MixedUnit& unit(int storage) {
 }
 }  // namespace
 
-// Upload the FP32 tables of every unit and opt the kernels into their shared memory.
+// Opt the kernels of every unit into their shared memory.
 cudaError_t prepare_mixed() {
-  cudaError_t e = upload_mixed_tables();  // this unit's copy, read by k_prepare_refs
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   for (int st : {ST_F32, ST_F32DEV, ST_BF16DEV, ST_F16DEV})
     if ((e = unit(st).prepare()) != cudaSuccess) return e;
   return cudaSuccess;

@@ -16,8 +16,7 @@
 // This header holds the kernels and their host helpers; each storage format is
 // instantiated in a translation unit of its own (rlbm_mixed_<storage>.cu) so
 // that the units compile in parallel, and rlbm_mixed.cu dispatches to them.
-// Every unit that includes it has its own copy of the constant tables and
-// uploads it (upload_mixed_tables) before its first launch.
+// Every unit that includes it has its own copy of the constant tables.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -28,23 +27,68 @@
 namespace rlbm {
 
 // ------------------------------------------------------------- FP32 tables
-static __constant__ float c_pf[3][6] = {RLBM_PF_MJ_INIT, RLBM_PF_FD_INIT, RLBM_PF_BE_INIT};
-static __constant__ float c_Qf[3][126] = {RLBM_QF_MJ_INIT, RLBM_QF_FD_INIT, RLBM_QF_BE_INIT};
-// exact defects of the FP32 tables in the conserved moments (see eq_moments)
-static __constant__ float c_Ef[3][18] = {RLBM_EF_MJ_INIT, RLBM_EF_FD_INIT, RLBM_EF_BE_INIT};
-static __constant__ float c_p2f[3][6];
-static __constant__ float c_pnkf[63];
-// terms of the power series of Li_nu(x), |x| <= 1/4
-#ifndef RLBM_SERIES_TERMS
-#define RLBM_SERIES_TERMS 12  // the first term left out is below 2^-24 of g_1 for |x| <= 1/4
-#endif
-constexpr int kSerF = RLBM_SERIES_TERMS, kExpBEf = 16, kExpFDf = 26;
-static __constant__ float c_invpowf[6 * kSerF];
-static __constant__ float c_be_expf[6 * kExpBEf];
-static __constant__ float c_fd_expf[6 * kExpFDf];
-static __constant__ float c_be_logcoeff[6];
-static __constant__ float c_be_harmf[6];
-static __constant__ float c_g_zcf[6];
+// terms of the power series of Li_nu(x), |x| <= 1/4 (the first one left out is below
+// 2^-24 of g_1), of the expansions in ln z, of the series in t = g_1 and of the
+// reversions t(w), t(G) (see solve_z_from_R)
+constexpr int kSerF = 12, kExpBEf = 16, kExpFDf = 26, kLogSerF = 9, kRevF = RLBM_NREV;
+
+// The FP64 tables rounded once to FP32 and laid out as the kernels read them, at
+// compile time: the constant bank holds them when the library is loaded, and creating
+// a handle uploads nothing.
+struct MixedTables {
+  float2 p[3][6];        // (p_s, p_s^2)
+  // projection by shell pair: Qp[EDF][j][i] = Q^(k)_{s n} of s = 2j and 2j + 1, i = n(n+1)/2 + k
+  float2 Qp[3][3][21];
+  float E[3][18];        // exact defects of the FP32 tables in the conserved moments (see eq_moments)
+  float2 invpow[3][kSerF];  // k^-nu of nu = 2i + 1, 2i + 2
+  float be_exp[6 * kExpBEf], fd_exp[6 * kExpFDf];
+  float be_logcoef[6], be_harm[6], g_zc[6];
+  float logser[5 * kLogSerF], rev[kRevF], revg[kRevF];
+};
+
+constexpr MixedTables make_mixed_tables() {
+  constexpr float pf[3][6] = {RLBM_PF_MJ_INIT, RLBM_PF_FD_INIT, RLBM_PF_BE_INIT};
+  constexpr double p2[3][6] = {RLBM_P2_MJ_INIT, RLBM_P2_FD_INIT, RLBM_P2_BE_INIT};
+  constexpr float Q[3][126] = {RLBM_QF_MJ_INIT, RLBM_QF_FD_INIT, RLBM_QF_BE_INIT};  // order k, s, n
+  constexpr float E[3][18] = {RLBM_EF_MJ_INIT, RLBM_EF_FD_INIT, RLBM_EF_BE_INIT};
+  constexpr double inv[6 * RLBM_NSERIES] = RLBM_INVPOW_INIT;
+  constexpr double be[6 * RLBM_NEXP] = RLBM_BE_EXP_INIT;
+  constexpr double fd[6 * RLBM_NEXP] = RLBM_FD_EXP_INIT;
+  constexpr double lc[6] = RLBM_BE_LOGCOEF_INIT, hm[6] = RLBM_BE_HARM_INIT, gz[6] = RLBM_G_ZC_INIT;
+  constexpr double ls[5 * RLBM_NLOGSER] = RLBM_LOGSER_INIT;
+  constexpr double rv[RLBM_NREV] = RLBM_REV_INIT, rg[RLBM_NREV] = RLBM_REVG_INIT;
+  MixedTables t{};
+  for (int e = 0; e < 3; ++e) {
+    for (int s = 0; s < 6; ++s) t.p[e][s] = float2{pf[e][s], (float)p2[e][s]};
+    for (int i = 0; i < 18; ++i) t.E[e][i] = E[e][i];
+    for (int j = 0; j < 3; ++j)
+      for (int n = 0; n < 6; ++n)
+        for (int k = 0; k <= n; ++k) {
+          const int o = qoff(k) + (n - k);
+          t.Qp[e][j][n * (n + 1) / 2 + k] = float2{Q[e][o + 2 * j * (6 - k)], Q[e][o + (2 * j + 1) * (6 - k)]};
+        }
+  }
+  for (int nu = 0; nu < 6; ++nu) {
+    for (int k = 0; k < kSerF; ++k) {
+      const float v = (float)inv[nu * RLBM_NSERIES + k];
+      if (nu % 2) t.invpow[nu / 2][k].y = v;
+      else t.invpow[nu / 2][k].x = v;
+    }
+    for (int k = 0; k < kExpBEf; ++k) t.be_exp[nu * kExpBEf + k] = (float)be[nu * RLBM_NEXP + k];
+    for (int k = 0; k < kExpFDf; ++k) t.fd_exp[nu * kExpFDf + k] = (float)fd[nu * RLBM_NEXP + k];
+    t.be_logcoef[nu] = (float)lc[nu];
+    t.be_harm[nu] = (float)hm[nu];
+    t.g_zc[nu] = (float)gz[nu];
+  }
+  for (int nu = 0; nu < 5; ++nu)
+    for (int k = 0; k < kLogSerF; ++k) t.logser[nu * kLogSerF + k] = (float)ls[nu * RLBM_NLOGSER + k];
+  for (int k = 0; k < kRevF; ++k) {
+    t.rev[k] = (float)rv[k];
+    t.revg[k] = (float)rg[k];
+  }
+  return t;
+}
+static __constant__ MixedTables c_mt = make_mixed_tables();
 
 constexpr float kPIf = 3.14159265358979f;
 // sqrt(3)/2 = kH + kHl: FP32 value and its residual. Products with sqrt(3)/2
@@ -60,19 +104,23 @@ constexpr float kRZCf = (float)RLBM_R_ZC;
 constexpr float kZCf = 0.9999999f;
 
 // --------------------------------------------------- FP32 EDF integrals g_nu
-// sum_{k>=1} x^k k^{-nu}, nu = 1..6, |x| <= 1/4. Fully unrolled, so that the
-// coefficients are immediate constant operands. Rolled, each term loaded its
+// sum_{k>=1} x^k k^{-nu}, nu = 1..6, |x| <= 1/4, two nu as a pair. Fully unrolled, so
+// that the coefficients are immediate constant operands. Rolled, each term loaded its
 // six coefficients first; unrolling made the FD and BE steps 14 % and 5 % faster.
 __device__ __forceinline__ void li_series6f(float x, float g[6]) {
-  float xk = 1.0f;
+  float xk = x;
+  f2 a[3];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) g[i] = 0.0f;
+  for (int i = 0; i < 3; ++i) a[i] = vmul(f2_dup(xk), f2_make(c_mt.invpow[i][0].x, c_mt.invpow[i][0].y));
 #pragma unroll
-  for (int k = 1; k <= kSerF; ++k) {
+  for (int k = 2; k <= kSerF; ++k) {
     xk *= x;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) g[i] = fmaf(xk, c_invpowf[i * kSerF + k - 1], g[i]);
+    for (int i = 0; i < 3; ++i)
+      a[i] = vfma(f2_dup(xk), f2_make(c_mt.invpow[i][k - 1].x, c_mt.invpow[i][k - 1].y), a[i]);
   }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) f2_split(a[i], g[2 * i], g[2 * i + 1]);
 }
 
 template <int EDF>
@@ -91,14 +139,14 @@ __device__ void g_allf(float z, float g[6]) {
 #pragma unroll 4
     for (int k = 0; k < kExpBEf; ++k) {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) g[i] = fmaf(mk, c_be_expf[i * kExpBEf + k], g[i]);
+      for (int i = 0; i < 6; ++i) g[i] = fmaf(mk, c_mt.be_exp[i * kExpBEf + k], g[i]);
       mk *= mu;
     }
     const float lnm = logf(-mu);
     float mp = 1.0f;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-      g[i] = fmaf(mp, fmaf(-c_be_logcoeff[i], lnm, c_be_harmf[i]), g[i]);
+      g[i] = fmaf(mp, fmaf(-c_mt.be_logcoef[i], lnm, c_mt.be_harm[i]), g[i]);
       mp *= mu;
     }
     return;
@@ -117,7 +165,7 @@ __device__ void g_allf(float z, float g[6]) {
 #pragma unroll 2
     for (int k = 0; k < kExpFDf; ++k) {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) g[i] = fmaf(mk, c_fd_expf[i * kExpFDf + k], g[i]);
+      for (int i = 0; i < 6; ++i) g[i] = fmaf(mk, c_mt.fd_exp[i * kExpFDf + k], g[i]);
       mk *= mu;
     }
     return;
@@ -141,14 +189,15 @@ template <int EDF>
 __device__ __forceinline__ void g123f(float z, float g[3]) {
   if (EDF != EDF_MJ && z <= 0.25f) {
     const float x = EDF == EDF_BE ? z : -z;
-    float xk = 1.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
+    float xk = x, s1, s2, s3 = xk * c_mt.invpow[1][0].x;
+    f2 a = vmul(f2_dup(xk), f2_make(c_mt.invpow[0][0].x, c_mt.invpow[0][0].y));
 #pragma unroll
-    for (int k = 1; k <= kSerF; ++k) {
+    for (int k = 2; k <= kSerF; ++k) {
       xk *= x;
-      s1 = fmaf(xk, c_invpowf[k - 1], s1);
-      s2 = fmaf(xk, c_invpowf[kSerF + k - 1], s2);
-      s3 = fmaf(xk, c_invpowf[2 * kSerF + k - 1], s3);
+      a = vfma(f2_dup(xk), f2_make(c_mt.invpow[0][k - 1].x, c_mt.invpow[0][k - 1].y), a);
+      s3 = fmaf(xk, c_mt.invpow[1][k - 1].x, s3);
     }
+    f2_split(a, s1, s2);
     const float sg = EDF == EDF_BE ? 1.0f : -1.0f;
     g[0] = sg * s1;
     g[1] = sg * s2;
@@ -174,6 +223,36 @@ __device__ __forceinline__ bool newton_done(float d, float z) {
   return d * d * cb < 1e-9f;
 }
 
+// The six g_nu of t = g_1 <= 0.5 (z = 0.65 FD, 0.39 BE): nine terms put the first one
+// left out below 1e-9 of the sum; no logarithm, no exponential (see g_all_t).
+template <int EDF>
+__device__ __forceinline__ void g_all_tf(float t, float g[6]) {
+  const float u = EDF == EDF_BE ? t : -t, u2 = u * u;
+  float a = c_mt.logser[8], b[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) b[j] = c_mt.logser[(j + 1) * kLogSerF + 8];
+  a = fmaf(fmaf(fmaf(a, u2, c_mt.logser[6]), u2, c_mt.logser[4]), u2, c_mt.logser[2]);  // odd ones vanish
+#pragma unroll
+  for (int n = 7; n >= 0; --n)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = fmaf(b[j], u, c_mt.logser[(j + 1) * kLogSerF + n]);
+  g[0] = t;
+  g[1] = t * fmaf(a, u2, fmaf(u, -0.25f, 1.0f));
+#pragma unroll
+  for (int j = 0; j < 4; ++j) g[2 + j] = t * b[j];
+}
+template <int EDF>
+__device__ __forceinline__ float z_of_tf(float t) { return EDF == EDF_BE ? -expm1f(-t) : expm1f(t); }
+// t = x sum_n a_n (s x)^n
+template <int EDF>
+__device__ __forceinline__ float revert_f(const float* c, float x) {
+  const float sx = EDF == EDF_BE ? x : -x;
+  float p = c[kRevF - 1];
+#pragma unroll
+  for (int n = kRevF - 2; n >= 0; --n) p = fmaf(p, sx, c[n]);
+  return x * p;
+}
+
 // Fugacity from g_3^2/g_2^3 = target (Eq. 25), FP32 safeguarded Newton in mu = ln z.
 // Start: the series g_nu = z + s z^2/2^nu + z^3/3^nu + s z^4/4^nu ... (s = -1 FD,
 // +1 BE) make w = 1/target = g_2^3/g_3^2 a power series in z; inverting it gives
@@ -182,11 +261,11 @@ __device__ __forceinline__ bool newton_done(float d, float z) {
 // it). The iterations evaluate g_1..g_3 alone; all six g_nu are evaluated once,
 // at the converged mu (the last step applied).
 template <int EDF>
-__device__ int solve_z_R_f(float target, float& z, float g[6]) {
+__device__ __forceinline__ int solve_z_R_newton_f(float target, float& z, float g[6]) {
   if (EDF == EDF_BE && target < kRZCf) {
     z = kZCf;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) g[i] = c_g_zcf[i];
+    for (int i = 0; i < 6; ++i) g[i] = c_mt.g_zc[i];
     return ST_CLAMPED;
   }
   float lo = -40.0f, hi = (EDF == EDF_BE) ? -1.0e-7f : 40.0f;
@@ -235,17 +314,12 @@ __device__ int solve_z_R_f(float target, float& z, float g[6]) {
 // theta^2)) gives mu = ln G +- G/4 - (5/288) G^2 +- G^3/288 + O(G^4) (upper signs
 // FD, lower BE) for small G. Convergence as in solve_z_R_f.
 template <int EDF>
-__device__ int solve_z_nt_f(float n, float theta, float& z, float g[6]) {
+__device__ __forceinline__ int solve_z_nt_newton_f(float n, float theta, float& z, float g[6]) {
   const float G = n / (2.0f * kPIf * theta * theta);
-  if (EDF == EDF_MJ) {
-    z = G;
-    g_allf<EDF>(z, g);
-    return 0;
-  }
-  if (EDF == EDF_BE && G >= c_g_zcf[1]) {
+  if (EDF == EDF_BE && G >= c_mt.g_zc[1]) {
     z = kZCf;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) g[i] = c_g_zcf[i];
+    for (int i = 0; i < 6; ++i) g[i] = c_mt.g_zc[i];
     return ST_CLAMPED;
   }
   float lo = -40.0f, hi = (EDF == EDF_BE) ? -1.0e-7f : 40.0f;
@@ -286,16 +360,84 @@ __device__ int solve_z_nt_f(float n, float theta, float& z, float g[6]) {
   return st;
 }
 
+// Fugacity of a cell from n and eps, by the Newton solve on the target ratio; with
+// kSeries (the 16-bit storages) from w = g_2^3/g_3^2 = (2/pi) n^3/eps^2. For w up to
+// 0.48 (z about 0.61 FD, 0.38 BE) ten terms of the reversion t(w) = w + (47/1728) w^3 + ...
+// give t to FP32 rounding (the first one left out is below 3e-9 of t) and g_all_tf
+// the g_nu; other states take the Newton solve, out of line. kZ: z is wanted.
+template <int EDF>
+__device__ __noinline__ int solve_z_R_other_f(float target, float& z, float g[6]) {
+  return solve_z_R_newton_f<EDF>(target, z, g);
+}
+template <int EDF>
+__device__ __noinline__ int solve_z_nt_other_f(float n, float theta, float& z, float g[6]) {
+  return solve_z_nt_newton_f<EDF>(n, theta, z, g);
+}
+template <int EDF, bool kSeries, bool kZ>
+__device__ __forceinline__ int solve_z_R_f(float n, float eps, float& z, float g[6]) {
+  const float target = 0.5f * kPIf * eps * eps / (n * n * n);
+  if constexpr (kSeries) {
+    const float w = (2.0f / kPIf) * (n * n * n) / (eps * eps);
+    if (w > 1e-30f && w < 0.48f) {
+      const float t = revert_f<EDF>(c_mt.rev, w);
+      g_all_tf<EDF>(t, g);
+      if (kZ) z = z_of_tf<EDF>(t);
+      return 0;
+    }
+    return solve_z_R_other_f<EDF>(target, z, g);
+  } else {
+    return solve_z_R_newton_f<EDF>(target, z, g);
+  }
+}
+
+// Fugacity from (n, theta): G = n / (2 pi theta^2) = g_2. The reversion t(G) converges
+// more slowly (ratio about G/2): ten terms reach FP32 rounding up to G = 0.25.
+template <int EDF, bool kSeries, bool kZ>
+__device__ __forceinline__ int solve_z_nt_f(float n, float theta, float& z, float g[6]) {
+  const float G = n / (2.0f * kPIf * theta * theta);
+  if constexpr (EDF == EDF_MJ) {
+    z = G;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) g[i] = G;
+    return 0;
+  } else if constexpr (kSeries) {
+    if (G > 1e-30f && G < 0.25f) {
+      const float t = revert_f<EDF>(c_mt.revg, G);
+      g_all_tf<EDF>(t, g);
+      if (kZ) z = z_of_tf<EDF>(t);
+      return 0;
+    }
+    return solve_z_nt_other_f<EDF>(n, theta, z, g);
+  } else {
+    return solve_z_nt_newton_f<EDF>(n, theta, z, g);
+  }
+}
+
 // ------------------------------------------------------------- Landau frame
+// Moments of a cell: N0, m = (T^01, T^02) and c = (N^1, N^2) (the reference state has
+// none), T^00 and the spatial stresses.
+struct MomentsDf {
+  df N0, T00, T11, T22;
+  f2 nv, m;   // (N^1, N^2), (T^01, T^02)
+  float T12;
+};
+
 // T^a_b U^b = eps U^a (Eq. 21) as m - Pi u = (T00 - m.u) u. FP32 Newton from the
 // ideal-fluid estimate, then one Newton correction whose residual is evaluated
 // in double-float (the FP32 Jacobian only scales the small correction), which
-// brings u to ~1e-15. eps, gamma follow in double-float. T = {T00, T01, T02,
-// T11, T12, T22}.
-__device__ __forceinline__ int landau_df(const df T[6], df& ux, df& uy, df& eps, df& gamma) {
+// brings u to ~1e-15. eps, gamma follow in double-float, |u|^2 and n on the way. The
+// x and y components run as one pair.
+struct FrameDf {
+  df2 u;
+  df eps, gamma, u2, n;
+};
+
+__device__ __forceinline__ int landau_df(const MomentsDf& M, FrameDf& F) {
   // every product that meets a sum is an explicit FMA (or the sum a rounded
   // intrinsic), so each kernel that inlines this gets the same roundings
-  const float E = T[0].hi, mx = T[1].hi, my = T[2].hi, pxx = T[3].hi, pxy = T[4].hi, pyy = T[5].hi;
+  float mx, my;
+  f2_split(M.m, mx, my);
+  const float E = M.T00.hi, pxx = M.T11.hi, pxy = M.T12, pyy = M.T22.hi;
   const float disc = fmaf(9.0f * E, E, -8.0f * fmaf(mx, mx, __fmul_rn(my, my)));
   if (!(E > 0.0f) || !(disc >= 0.0f)) return ST_NONPHYSICAL;
   const float x = 0.25f * fmaf(3.0f, E, sqrtf(disc));
@@ -312,86 +454,116 @@ __device__ __forceinline__ int landau_df(const df T[6], df& ux, df& uy, df& eps,
     fv = fmaf(fmaf(j10, fx, -__fmul_rn(j00, fy)), rdet, fv);
   }
   if (!(fmaf(fu, fu, __fmul_rn(fv, fv)) < 1.0f)) return ST_NONPHYSICAL;
+  const f2 f = f2_make(fu, fv);
   {
-    const df a = df_sub(T[0], df_add(df_mul(T[1], fu), df_mul(T[2], fv)));
-    const df rx = df_sub(df_sub(T[1], df_add(df_mul(T[3], fu), df_mul(T[4], fv))), df_mul(a, fu));
-    const df ry = df_sub(df_sub(T[2], df_add(df_mul(T[4], fu), df_mul(T[5], fv))), df_mul(a, fv));
+    const df2 mf = two_prod(M.m, f);
+    const df a = df_sub(M.T00, df_add(df_first(mf), df_second(mf)));
+    const df2 pu = df_add(df_mul(df_make(f2_make(M.T11.hi, pxy), f2_make(M.T11.lo, 0.0f)), f2_dup(fu)),
+                          df_mul(df_make(f2_make(pxy, M.T22.hi), f2_make(0.0f, M.T22.lo)), f2_dup(fv)));
+    const df2 r = df_sub(df_add(df_neg(pu), M.m), df_mul(df_dup(a), f));
     const float af = a.hi;
     const float j00 = __fsub_rn(fmaf(fu, mx, -pxx), af), j01 = fmaf(fu, my, -pxy), j10 = fmaf(fv, mx, -pxy),
                 j11 = __fsub_rn(fmaf(fv, my, -pyy), af);
     const float rdet = 1.0f / fmaf(j00, j11, -__fmul_rn(j01, j10));
-    const float gx = df_to_float(rx), gy = df_to_float(ry);
-    ux = two_sum(fu, __fmul_rn(fmaf(j01, gy, -__fmul_rn(j11, gx)), rdet));
-    uy = two_sum(fv, __fmul_rn(fmaf(j10, gx, -__fmul_rn(j00, gy)), rdet));
+    float gx, gy;
+    f2_split(df_to_float(r), gx, gy);
+    F.u = two_sum(f, f2_make(__fmul_rn(fmaf(j01, gy, -__fmul_rn(j11, gx)), rdet),
+                             __fmul_rn(fmaf(j10, gx, -__fmul_rn(j00, gy)), rdet)));
   }
-  eps = df_sub(T[0], df_add(df_mul(T[1], ux), df_mul(T[2], uy)));
-  const df w = df_sub(df_make(1.0f, 0.0f), df_add(df_mul(ux, ux), df_mul(uy, uy)));
-  if (!(w.hi > 0.0f) || !(eps.hi > 0.0f)) return ST_NONPHYSICAL;
-  gamma = df_rsqrt(w);
+  const df2 mu = df_mul(F.u, M.m), uu = df_mul(F.u, F.u), nu = df_mul(F.u, M.nv);
+  F.eps = df_sub(M.T00, df_add(df_first(mu), df_second(mu)));
+  F.u2 = df_add(df_first(uu), df_second(uu));
+  const df w = df_sub(df_make(1.0f, 0.0f), F.u2);
+  if (!(w.hi > 0.0f) || !(F.eps.hi > 0.0f)) return ST_NONPHYSICAL;
+  F.gamma = df_rsqrt(w);
+  F.n = df_mul(F.gamma, df_sub(M.N0, df_add(df_first(nu), df_second(nu))));
+  if (!(F.n.hi > 0.0f) || !isfinite(F.n.hi)) return ST_NONPHYSICAL;
   return 0;
 }
 
-// Relaxation rate of direction d, gamma (1 - v_d . u) / tau (Eq. 3), with the
-// roundings written out (see landau_df).
-__device__ __forceinline__ float relax_rate(int d, float gam, float ux, float uy, float itau) {
-  const float vu = fmaf((float)dcos(d), ux, __fmul_rn((float)dsin(d), uy));
-  return __fmul_rn(__fmul_rn(gam, __fsub_rn(1.0f, vu)), itau);
-}
-
-// FP32 harmonic sums of a 12-vector (pairs d, d+6 folded first).
-struct HarmF {
-  float h0, c1, s1, c2, s2;
-};
-
-__device__ __forceinline__ HarmF harmonics_f(const float v[12]) {
-  float e[6], o[6];
+// FP32 harmonic sums of the per-direction sums (A_d, B_d), the two kinds as a pair
+// (directions d, d + 6 folded first), and the moment totals in double-float:
+// reference moments + FP32 deviation sums.
+__device__ __forceinline__ MomentsDf moments_df(const DomDev& D, const f2 v[12]) {
+  const f2 half = f2_dup(0.5f), h = f2_dup(kH), hl = f2_dup(kHl);
+  f2 e[6], o[6];
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
-    e[d] = v[d] + v[d + 6];
-    o[d] = v[d] - v[d + 6];
+    e[d] = vadd(v[d], v[d + 6]);
+    o[d] = vsub(v[d], v[d + 6]);
   }
-  HarmF H;
-  H.h0 = ((e[0] + e[1]) + (e[2] + e[3])) + (e[4] + e[5]);
-  H.c1 = fma_h(o[1] - o[5], fmaf(0.5f, o[2] - o[4], o[0]));
-  H.s1 = fma_h(o[2] + o[4], fmaf(0.5f, o[1] + o[5], o[3]));
-  H.c2 = fmaf(0.5f, (e[1] - e[2]) + (e[5] - e[4]), e[0] - e[3]);
-  H.s2 = mul_h((e[1] + e[2]) - (e[4] + e[5]));
-  return H;
+  const f2 h0 = vadd(vadd(vadd(e[0], e[1]), vadd(e[2], e[3])), vadd(e[4], e[5]));
+  const f2 c1x = vsub(o[1], o[5]), s1x = vadd(o[2], o[4]);
+  const f2 c1 = vfma(h, c1x, vfma(hl, c1x, vfma(half, vsub(o[2], o[4]), o[0])));
+  const f2 s1 = vfma(h, s1x, vfma(hl, s1x, vfma(half, vadd(o[1], o[5]), o[3])));
+  float be[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) be[d] = f2_hi(e[d]);
+  const float c2 = fmaf(0.5f, __fadd_rn(__fsub_rn(be[1], be[2]), __fsub_rn(be[5], be[4])), __fsub_rn(be[0], be[3]));
+  const float s2 = mul_h(__fsub_rn(__fadd_rn(be[1], be[2]), __fadd_rn(be[4], be[5])));
+  MomentsDf M;
+  M.N0 = df_add(df_make(D.n0_hl[0], D.n0_hl[1]), f2_lo(h0));
+  M.T00 = df_add(df_make(D.t00_hl[0], D.t00_hl[1]), f2_hi(h0));
+  M.nv = f2_make(f2_lo(c1), f2_lo(s1));
+  M.m = f2_make(f2_hi(c1), f2_hi(s1));
+  M.T11 = df_scale(df_add(M.T00, c2), 0.5f);
+  M.T12 = 0.5f * s2;
+  M.T22 = df_scale(df_add(M.T00, -c2), 0.5f);
+  return M;
 }
 
-// FP32 deviation of the equilibrium from fref for shell s (12 directions):
-// R^{c|s}_k = sum_n Qf^(k)_{s n} dZ_nk (+ rres_s in R^c_0), then the folded
-// 12-point synthesis (same symmetries as the FP64 form).
+// Relaxation rates gamma (1 - v_d . u) / tau (Eq. 3), the directions d and d + 6
+// (v_d . u of opposite sign) as a pair, with the roundings written out (see landau_df).
+__device__ __forceinline__ void relax_rates(float gam, float ux, float uy, float itau, float om[12]) {
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const float vu = fmaf((float)dcos(d), ux, __fmul_rn((float)dsin(d), uy));
+    f2_split(vmul(vmul(f2_dup(gam), vsub(f2_dup(1.0f), f2_make(vu, -vu))), f2_dup(itau)), om[d], om[d + 6]);
+  }
+}
+
+// Equilibrium-moment deviations dZ_nk = Z_nk - Z_ref, Re and Im, indexed n(n+1)/2 + k.
+struct EqF {
+  float zr[21], zi[21];
+};
+
+// FP32 deviation of the equilibrium from fref for the shells s = 2j, 2j + 1 (12
+// directions, the two shells as a pair): R^{c|s}_k = sum_n Q^(k)_{s n} dZ_nk (+ rres_s in
+// R^c_0), then the folded 12-point synthesis (same symmetries as the FP64 form). The
+// harmonics carry the powers of u before the projection: the momentum of the
+// equilibrium is a sum of Q Z_n1, whose rounding must vary from cell to cell with u
+// (rounded as one constant factor times u it would be off by the same 3e-8 in every
+// cell and step, a steady source of momentum).
 template <int EDF>
-__device__ __forceinline__ void dfeq_shell(int s, float rres, const float zr[21], const float zi[21],
-                                           float fe[12]) {
-  float Rc[6], Rs[6];
+__device__ __forceinline__ void dfeq_pair(int j, f2 rres, const EqF& q, f2 fe[12]) {
+  f2 Rc[6], Rs[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    float ac = 0.0f, as = 0.0f;
 #pragma unroll
     for (int n = k; n < 6; ++n) {
-      const float q = c_Qf[EDF][qoff(k) + s * (6 - k) + (n - k)];
-      ac = fmaf(q, zr[n * (n + 1) / 2 + k], ac);
-      as = fmaf(q, zi[n * (n + 1) / 2 + k], as);
+      const int i = n * (n + 1) / 2 + k;
+      const f2 t = f2_make(c_mt.Qp[EDF][j][i].x, c_mt.Qp[EDF][j][i].y);
+      Rc[k] = n == k ? vmul(t, f2_dup(q.zr[i])) : vfma(t, f2_dup(q.zr[i]), Rc[k]);
+      if (k) Rs[k] = n == k ? vmul(t, f2_dup(q.zi[i])) : vfma(t, f2_dup(q.zi[i]), Rs[k]);
     }
-    Rc[k] = ac;
-    Rs[k] = as;
   }
-  Rc[0] += rres;
-  const float t1 = Rc[0] + Rc[4], t2 = fmaf(-0.5f, Rc[4], Rc[0]);
-  const float Ec0 = t1 + Rc[2], Ec3 = t1 - Rc[2], Ec1 = fmaf(0.5f, Rc[2], t2), Ec2 = fmaf(-0.5f, Rc[2], t2);
-  const float Es1 = mul_h(Rs[2] + Rs[4]), Es2 = mul_h(Rs[2] - Rs[4]);
-  const float E0 = Ec0, E1 = Ec1 + Es1, E2 = Ec2 + Es2, E3 = Ec3, E4 = Ec2 - Es2, E5 = Ec1 - Es1;
-  const float Oc0 = Rc[1] + Rc[3] + Rc[5], Oc1 = mul_h(Rc[1] - Rc[5]), Oc2 = fmaf(0.5f, Rc[1] + Rc[5], -Rc[3]);
-  const float Os1 = fmaf(0.5f, Rs[1] + Rs[5], Rs[3]), Os2 = mul_h(Rs[1] - Rs[5]), Os3 = Rs[1] - Rs[3] + Rs[5];
-  const float O0 = Oc0, O1 = Oc1 + Os1, O2 = Oc2 + Os2, O3 = Os3, O4 = Os2 - Oc2, O5 = Os1 - Oc1;
-  fe[0] = E0 + O0; fe[6] = E0 - O0;
-  fe[1] = E1 + O1; fe[7] = E1 - O1;
-  fe[2] = E2 + O2; fe[8] = E2 - O2;
-  fe[3] = E3 + O3; fe[9] = E3 - O3;
-  fe[4] = E4 + O4; fe[10] = E4 - O4;
-  fe[5] = E5 + O5; fe[11] = E5 - O5;
+  Rc[0] = vadd(Rc[0], rres);
+  const f2 half = f2_dup(0.5f), mhalf = f2_dup(-0.5f), h = f2_dup(kH), hl = f2_dup(kHl);
+  auto mulh = [&](f2 x) { return vfma(h, x, vmul(hl, x)); };
+  const f2 t1 = vadd(Rc[0], Rc[4]), t2 = vfma(mhalf, Rc[4], Rc[0]);
+  const f2 Ec0 = vadd(t1, Rc[2]), Ec3 = vsub(t1, Rc[2]), Ec1 = vfma(half, Rc[2], t2), Ec2 = vfma(mhalf, Rc[2], t2);
+  const f2 Es1 = mulh(vadd(Rs[2], Rs[4])), Es2 = mulh(vsub(Rs[2], Rs[4]));
+  const f2 E[6] = {Ec0, vadd(Ec1, Es1), vadd(Ec2, Es2), Ec3, vsub(Ec2, Es2), vsub(Ec1, Es1)};
+  const f2 Oc0 = vadd(vadd(Rc[1], Rc[3]), Rc[5]), Oc1 = mulh(vsub(Rc[1], Rc[5])),
+           Oc2 = vfma(half, vadd(Rc[1], Rc[5]), vneg(Rc[3]));
+  const f2 Os1 = vfma(half, vadd(Rs[1], Rs[5]), Rs[3]), Os2 = mulh(vsub(Rs[1], Rs[5])),
+           Os3 = vadd(vsub(Rs[1], Rs[3]), Rs[5]);
+  const f2 O[6] = {Oc0, vadd(Oc1, Os1), vadd(Oc2, Os2), Os3, vsub(Os2, Oc2), vsub(Os1, Oc1)};
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    fe[d] = vadd(E[d], O[d]);
+    fe[d + 6] = vsub(E[d], O[d]);
+  }
 }
 
 // FP32 equilibrium-moment deviations dZ_nk = Z_nk - Z_ref (Appendix, harmonic
@@ -400,69 +572,102 @@ __device__ __forceinline__ void dfeq_shell(int s, float rres, const float zr[21]
 // the conserved isotropic entries dZ_10, dZ_20 itself.
 template <int EDF>
 __device__ __forceinline__ void dz_moments(const DomDev& D, const float g[6], float theta, float ux, float uy,
-                                           float gam, float An1, float An2, float zr[21], float zi[21]) {
+                                           float gam, float An1, float An2, EqF& q) {
   // products that meet sums are explicit FMAs (see landau_df)
   const float u2 = fmaf(ux, ux, __fmul_rn(uy, uy));
   float wr[6], wi[6];
-  wr[0] = 1.0f;
-  wi[0] = 0.0f;
+  wr[1] = ux;
+  wi[1] = uy;
 #pragma unroll
-  for (int k = 1; k < 6; ++k) {
+  for (int k = 2; k < 6; ++k) {
     wr[k] = fmaf(wr[k - 1], ux, -__fmul_rn(wi[k - 1], uy));
     wi[k] = fmaf(wr[k - 1], uy, __fmul_rn(wi[k - 1], ux));
   }
   float A = 2.0f * kPIf * theta;
 #pragma unroll
   for (int n = 0; n < 6; ++n) {
-    if (n > 0) A *= (float)n * theta * gam;
-    float An = A * g[n];
+    if (n > 0) A = __fmul_rn(A, __fmul_rn(__fmul_rn((float)n, theta), gam));
+    float An = __fmul_rn(A, g[n]);  // (a plain product would be contracted where P is 1)
     if (n == 1 && An1 >= 0.0f) An = An1;
     if (n == 2 && An2 >= 0.0f) An = An2;
 #pragma unroll
     for (int k = 0; k <= n; ++k) {
       const int i = n * (n + 1) / 2 + k;
-      const float P = fmaf(u2, fmaf(u2, c_pnkf[3 * i + 2], c_pnkf[3 * i + 1]), c_pnkf[3 * i + 0]);
+      const float p0 = (float)pnk(3 * i), p1 = (float)pnk(3 * i + 1), p2 = (float)pnk(3 * i + 2);
+      const float P = p2 != 0.0f ? fmaf(u2, fmaf(u2, p2, p1), p0) : (p1 != 0.0f ? fmaf(u2, p1, p0) : p0);
       if (k == 0) {
-        zr[i] = fmaf(An, P, -D.zref_f[n]);  // the isotropic moments as deviations from the reference
-        zi[i] = 0.0f;
+        q.zr[i] = fmaf(An, P, -D.zref_f[n]);  // the isotropic moments as deviations from the reference
       } else {
         const float sc = __fmul_rn(An, P);
-        zr[i] = __fmul_rn(sc, wr[k]);
-        zi[i] = __fmul_rn(sc, wi[k]);
+        q.zr[i] = __fmul_rn(sc, wr[k]);
+        q.zi[i] = __fmul_rn(sc, wi[k]);
       }
     }
   }
 }
 
+// Remove the FP32 tables' defects in N^0, T^00, T^0x, T^0y (FP32 suffices: the
+// corrections are ~1e-8 of the moments).
+template <int EDF>
+__device__ __forceinline__ void remove_defects(EqF& q) {
+  float d10 = 0.0f, d20 = 0.0f, d21r = 0.0f, d21i = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    d10 = fmaf(c_mt.E[EDF][k], q.zr[k * (k + 1) / 2], d10);
+    d20 = fmaf(c_mt.E[EDF][6 + k], q.zr[k * (k + 1) / 2], d20);
+  }
+#pragma unroll
+  for (int k = 1; k < 6; ++k) {
+    d21r = fmaf(c_mt.E[EDF][12 + k], q.zr[k * (k + 1) / 2 + 1], d21r);
+    d21i = fmaf(c_mt.E[EDF][12 + k], q.zi[k * (k + 1) / 2 + 1], d21i);
+  }
+  q.zr[1] = __fsub_rn(q.zr[1], d10);
+  q.zr[3] = __fsub_rn(q.zr[3], d20);
+  q.zr[4] = __fsub_rn(q.zr[4], d21r);
+  q.zi[4] = __fsub_rn(q.zi[4], d21i);
+}
+
+// Equilibrium deviations of a shell pair in work units (see the storage policies).
+template <int EDF, class S>
+__device__ __forceinline__ void dfeq_work(const DomDev& D, int j, const EqF& q, f2 fe[12]) {
+  dfeq_pair<EDF>(j, f2_make(D.rres[2 * j], D.rres[2 * j + 1]), q, fe);
+  if constexpr (S::kScaled) {
+    const f2 b = f2_make(D.b_s[2 * j], D.b_s[2 * j + 1]);
+#pragma unroll
+    for (int d = 0; d < 12; ++d) fe[d] = vmul(b, fe[d]);
+  }
+}
+
 // Halo writer of the mixed step: copies of the cell's post-collision values
-// (FP32 deviations held in its shared-memory column col[q * kThreads]) and, at
+// (work units, held in its shared-memory column col[pair * kThreads]) and, at
 // fixed-T walls, the
 // FP32 equilibrium deviation of the wall ghost. Reading the copies back from
 // global memory instead would put a read-after-write round trip to L2 on every
 // edge warp, which costs more than keeping the column up to date.
 template <int EDF, class S>
 __device__ __noinline__ void write_halo_mixed(const DomDev& D, int x, int y, typename S::T* __restrict__ fout,
-                                              const float* col, bool have_state, float n, float ux, float uy,
+                                              const f2* col, bool have_state, float n, float ux, float uy,
                                               float gam, unsigned& st, bool images) {
+  using P = Pair<typename S::T>;
   int hx[8], hy[8], wall[8];
   const int cnt = halo_targets(D, x, y, hx, hy, wall, images);
   for (int i = 0; i < cnt; ++i) {
-    const long long h = cell_rel(D, hx[i], hy[i]);
+    typename S::T* h = fout + cell_rel(D, hx[i], hy[i]);
     if (wall[i] < 0 || !have_state) {
-      for (int q = 0; q < 72; ++q) {
-        fout[q * kBlkW + h] = S::encf(col[q * kThreads], D, q % 6);
-      }
+      for (int k = 0; k < kPairs; ++k)
+        *reinterpret_cast<P*>(h + k * kSegW) = S::enc2(col[k * kThreads], D, 2 * (k % 3));
     } else {
       const float tw = D.t_wall_f[wall[i]];
       float z, g[6];
-      st |= solve_z_nt_f<EDF>(n, tw, z, g);
-      float zr[21], zi[21];
-      dz_moments<EDF>(D, g, tw, ux, uy, gam, -1.0f, -1.0f, zr, zi);
+      st |= solve_z_nt_f<EDF, S::kScaled, false>(n, tw, z, g);
+      EqF q;
+      dz_moments<EDF>(D, g, tw, ux, uy, gam, -1.0f, -1.0f, q);
 #pragma unroll 1
-      for (int s = 0; s < 6; ++s) {
-        float fe[12];
-        dfeq_shell<EDF>(s, D.rres[s], zr, zi, fe);
-        for (int d = 0; d < 12; ++d) fout[(6 * d + s) * kBlkW + h] = S::encf(fe[d], D, s);
+      for (int j = 0; j < 3; ++j) {
+        f2 fe[12];
+        dfeq_work<EDF, S>(D, j, q, fe);
+#pragma unroll
+        for (int d = 0; d < 12; ++d) *reinterpret_cast<P*>(h + (3 * d + j) * kSegW) = S::enc2(fe[d], D, 2 * j);
       }
     }
   }
@@ -470,48 +675,48 @@ __device__ __noinline__ void write_halo_mixed(const DomDev& D, int x, int y, typ
 
 constexpr size_t kSmemF = 72 * kThreads * sizeof(float);  // the shared-memory column of a block
 
-#ifndef RLBM_MIXED_MIN_BLOCKS
-// resident blocks per SM the register budget must allow: 640 threads (96
-// registers, no spills; 20 warps per SM). Measured against 512 threads (128
-// registers) and 768 (80 registers, spills): 2 % faster than the first on every
-// workload, 12 % faster than the second.
-#define RLBM_MIXED_MIN_BLOCKS (640 / kThreads)
-#endif
+// Resident blocks of 128 threads per SM that the register budget must allow: 5 (96
+// registers, 20 warps) for the FP32 storages without halo work, 4 (128 registers, 16
+// warps) for the 16-bit ones and wherever the halo writer's arguments would spill.
+// Measured, 5 against 4 blocks, MLUPS: 2048^2 FP32 deviations 11,096 / 10,919, 128-domain
+// batch 10,734 / 10,514; the batch in FP16 12,322 / 12,600; FD Fourier batch with
+// walls in BF16 8,558 / 10,427, in FP32 deviations 8,311 / 9,557.
+template <class S, int kHalo>
+constexpr int mixed_min_blocks() {
+  return (kHalo == 0 && !S::kScaled ? 640 : 512) / kThreads;
+}
 // 1: at the start of a tile one thread asks L2 for the tile's own blocks in rows
 // y0-1 .. y0+kTileH (one contiguous segment per row), so that the pull's later
 // directions find them in L2
 #ifndef RLBM_MIXED_L2_PREFETCH
 #define RLBM_MIXED_L2_PREFETCH 1
 #endif
-// 1: only warps holding an edge cell keep the relaxed values in the column (a
-// second copy of the relaxation loop); 0: every warp keeps them (one loop)
-#ifndef RLBM_MIXED_EDGE_WARPS
-#define RLBM_MIXED_EDGE_WARPS 0
-#endif
 
-// Relaxation (Eq. 3) of one cell's 72 pulled deviations in its column, shell
-// by shell, stored to fout; kKeep: the relaxed values also go back into the
-// column (warps holding an edge cell, whose halo writer reads them there).
+// Relaxation (Eq. 3) of one cell's 72 pulled deviations in its column, a shell pair
+// at a time (unrolled: the tables are immediate operands, 5 % faster than a loop),
+// stored to fout; kKeep: the relaxed values also go back into the
+// column (the halo writer reads them there).
 template <int EDF, class S, bool kKeep>
-__device__ __forceinline__ void relax_cell(const DomDev& D, const float zr[21], const float zi[21], const float om[12],
-                                           float* smf, int tid, long long c, typename S::T* __restrict__ fout) {
-#pragma unroll 1
-  for (int s = 0; s < 6; ++s) {
-    float fe[12];
-    dfeq_shell<EDF>(s, D.rres[s], zr, zi, fe);
+__device__ __forceinline__ void relax_cell(const DomDev& D, const EqF& q, const float om[12], f2* col,
+                                           typename S::T* __restrict__ out) {
+  using P = Pair<typename S::T>;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    f2 fe[12];
+    dfeq_work<EDF, S>(D, j, q, fe);
 #pragma unroll
     for (int d = 0; d < 12; ++d) {
-      const int q = 6 * d + s;
-      const float v = smf[q * kThreads + tid];
-      const float r = fmaf(om[d], fe[d] - v, v);
-      if constexpr (kKeep) smf[q * kThreads + tid] = r;
-      fout[q * kBlkW + c] = S::encf(r, D, s);
+      const int k = 3 * d + j;
+      const f2 v = col[k * kThreads];
+      const f2 r = vfma(f2_dup(om[d]), vsub(fe[d], v), v);
+      if constexpr (kKeep) col[k * kThreads] = r;
+      *reinterpret_cast<P*>(out + k * kSegW) = S::enc2(r, D, 2 * j);
     }
   }
 }
 
-// Collision of one cell (Eqs. 20-25, 10-11 and 3) from its pulled FP32
-// deviations, held in the thread's shared-memory column smf[q * kThreads + tid],
+// Collision of one cell (Eqs. 20-25, 10-11 and 3) from its pulled values in work
+// units, held in the thread's shared-memory column col[pair * kThreads],
 // and the shell sums A_d = sum_s p_s dv_{6d+s}, B_d = sum_s p_s^2 dv_{6d+s} of
 // each direction; stores f* to fout, writes the cell's halo images and returns
 // its status bits. Called by the active lanes of a warp (the lanes of cells
@@ -522,9 +727,8 @@ __device__ __forceinline__ void relax_cell(const DomDev& D, const float zr[21], 
 // sides). Below 2, with kImages = false, no halo cell copies the cell's relaxed
 // values, so they need not go back to the column.
 template <int EDF, class S, bool kImages, int kHalo = 2>
-__device__ __forceinline__ unsigned collide_mixed(const DomDev& D, int x, int y, long long c, const float A[12],
-                                                  const float B[12], float* smf, int tid,
-                                                  typename S::T* __restrict__ fout) {
+__device__ __forceinline__ unsigned collide_mixed(const DomDev& D, int x, int y, long long c, const f2 AB[12],
+                                                  f2* col, typename S::T* __restrict__ fout) {
   // a warp with no cell on an edge that has halo cells to write skips the halo
   // writer (uniform per warp)
   const bool edge = kImages ? (x == 0 || x == D.nx - 1 || y == 0 || y == D.ny - 1)
@@ -533,28 +737,16 @@ __device__ __forceinline__ unsigned collide_mixed(const DomDev& D, int x, int y,
                                         (y == 0 && bc_writes_halo(D.bc[2])) ||
                                         (y == D.ny - 1 && bc_writes_halo(D.bc[3])));
   const bool edge_warp = __any_sync(__activemask(), edge);
-  const HarmF ha = harmonics_f(A), hb = harmonics_f(B);
-  // moment totals in double-float: reference moments + FP32 deviation sums
-  const df N0 = df_add(df_make(D.n0_hl[0], D.n0_hl[1]), ha.h0);
-  const df H0 = df_add(df_make(D.t00_hl[0], D.t00_hl[1]), hb.h0);
-  df T[6];
-  T[0] = H0;
-  T[1] = df_make(hb.c1, 0.0f);
-  T[2] = df_make(hb.s1, 0.0f);
-  T[3] = df_scale(df_add(H0, hb.c2), 0.5f);
-  T[4] = df_make(0.5f * hb.s2, 0.0f);
-  T[5] = df_scale(df_add(H0, -hb.c2), 0.5f);
-  df ux, uy, eps, gam;
-  unsigned st = landau_df(T, ux, uy, eps, gam);
-  df n = df_make(0.0f, 0.0f);
-  if (!(st & ST_NONPHYSICAL)) {
-    n = df_mul(gam, df_sub(N0, df_add(df_mul(ux, ha.c1), df_mul(uy, ha.s1))));
-    if (!(n.hi > 0.0f) || !isfinite(n.hi)) st |= ST_NONPHYSICAL;
-  }
+  const MomentsDf M = moments_df(D, AB);
+  FrameDf F;
+  unsigned st = landau_df(M, F);
   const bool ok = !(st & ST_NONPHYSICAL);
-  const float uxf = df_to_float(ux), uyf = df_to_float(uy), gf = df_to_float(gam), nf = df_to_float(n);
+  float uxf = 0.0f, uyf = 0.0f, gf = 0.0f, nf = 0.0f;
   if (ok) {
-    const float ef = df_to_float(eps);
+    f2_split(df_to_float(F.u), uxf, uyf);
+    gf = df_to_float(F.gamma);
+    nf = df_to_float(F.n);
+    const float ef = df_to_float(F.eps);
     float theta, z, g[6];
     if (EDF == EDF_MJ) {
       theta = ef / (2.0f * nf);
@@ -562,8 +754,7 @@ __device__ __forceinline__ unsigned collide_mixed(const DomDev& D, int x, int y,
 #pragma unroll
       for (int i = 0; i < 6; ++i) g[i] = z;
     } else {
-      const float target = 0.5f * kPIf * ef * ef / (nf * nf * nf);
-      const int zs = solve_z_R_f<EDF>(target, z, g);
+      const int zs = solve_z_R_f<EDF, S::kScaled, false>(nf, ef, z, g);
       st |= zs;
       if (zs & ST_CLAMPED) theta = sqrtf(nf / (2.0f * kPIf * g[1]));
       else theta = 0.5f * g[1] / g[2] * ef / nf;
@@ -571,61 +762,60 @@ __device__ __forceinline__ unsigned collide_mixed(const DomDev& D, int x, int y,
     // conserved equilibrium moments from the double-float state: Z_1k from
     // n gamma, Z_2k from eps gamma^2 (a clamped BE state relaxes to its own
     // equilibrium energy 4 pi theta^3 g_3(z_c))
-    const df nG = df_mul(n, gam);
-    df eG2 = df_mul(df_mul(eps, gam), gam);
+    const df2 ne = df_mul(df_join(F.n, F.eps), df_dup(F.gamma));
+    const df nG = df_first(ne);
+    df eG2 = df_mul(df_second(ne), F.gamma);
     if (st & ST_CLAMPED) eG2 = df_make(4.0f * kPIf * theta * theta * theta * g[2] * gf * gf, 0.0f);
-    float zr[21], zi[21];
-    dz_moments<EDF>(D, g, theta, uxf, uyf, gf, nG.hi, eG2.hi, zr, zi);
+    EqF q;
+    dz_moments<EDF>(D, g, theta, uxf, uyf, gf, nG.hi, eG2.hi, q);
     // Z_20 = eps gamma^2 (1 + u^2/2), all in double-float
-    const df u2h = df_scale(df_add(df_mul(ux, ux), df_mul(uy, uy)), 0.5f);
     const df dz10 = df_sub(nG, df_make(D.z1_hl[0], D.z1_hl[1]));
-    const df dz20 = df_sub(df_add(eG2, df_mul(eG2, u2h)), df_make(D.z2_hl[0], D.z2_hl[1]));
-    zr[1] = df_to_float(dz10);
-    zr[3] = df_to_float(dz20);
+    const df dz20 = df_sub(df_add(eG2, df_mul(eG2, df_scale(F.u2, 0.5f))), df_make(D.z2_hl[0], D.z2_hl[1]));
+    q.zr[1] = df_to_float(dz10);
+    q.zr[3] = df_to_float(dz20);
     // Z_21 = (3/2) eps gamma^2 (u_x + i u_y) (Appendix; the rest state has none),
     // also from the double-float state rather than from FP32 eps gamma^2
-    const df e15 = df_mul(eG2, 1.5f);
-    zr[4] = df_to_float(df_mul(e15, ux));
-    zi[4] = df_to_float(df_mul(e15, uy));
-    // remove the FP32 tables' defects in N^0, T^00, T^0x, T^0y (FP32 suffices:
-    // the corrections are ~1e-8 of the moments)
-    float d10 = 0.0f, d20 = 0.0f, d21r = 0.0f, d21i = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      d10 = fmaf(c_Ef[EDF][k], zr[k * (k + 1) / 2], d10);
-      d20 = fmaf(c_Ef[EDF][6 + k], zr[k * (k + 1) / 2], d20);
-    }
-#pragma unroll
-    for (int k = 1; k < 6; ++k) {
-      d21r = fmaf(c_Ef[EDF][12 + k], zr[k * (k + 1) / 2 + 1], d21r);
-      d21i = fmaf(c_Ef[EDF][12 + k], zi[k * (k + 1) / 2 + 1], d21i);
-    }
-    zr[1] -= d10;
-    zr[3] -= d20;
-    zr[4] -= d21r;
-    zi[4] -= d21i;
+    f2_split(df_to_float(df_mul(df_dup(df_mul(eG2, 1.5f)), F.u)), q.zr[4], q.zi[4]);
+    remove_defects<EDF>(q);
     // constant tau, or the local tau = 4 (eta/s) / theta + 0.2546 of Sec. 3.5
     float itau = D.inv_tau_f;
     if (D.eta_s_f > 0.0f) itau = 1.0f / (4.0f * D.eta_s_f / theta + 0.2546f);
     float om[12];
-#pragma unroll
-    for (int d = 0; d < 12; ++d) om[d] = relax_rate(d, gf, uxf, uyf, itau);
-    if constexpr (!kImages && kHalo < 2) {
-      relax_cell<EDF, S, false>(D, zr, zi, om, smf, tid, c, fout);
-    } else {
-#if RLBM_MIXED_EDGE_WARPS
-      if (edge_warp) relax_cell<EDF, S, true>(D, zr, zi, om, smf, tid, c, fout);
-      else relax_cell<EDF, S, false>(D, zr, zi, om, smf, tid, c, fout);
-#else
-      relax_cell<EDF, S, true>(D, zr, zi, om, smf, tid, c, fout);
-#endif
-    }
+    relax_rates(gf, uxf, uyf, itau, om);
+    relax_cell<EDF, S, kImages || kHalo == 2>(D, q, om, col, fout + c);
   } else {
-    for (int q = 0; q < 72; ++q) fout[q * kBlkW + c] = S::encf(smf[q * kThreads + tid], D, q % 6);
+    for (int k = 0; k < kPairs; ++k)
+      *reinterpret_cast<Pair<typename S::T>*>(fout + c + k * kSegW) = S::enc2(col[k * kThreads], D, 2 * (k % 3));
   }
   if (kImages || kHalo > 0)
-    if (edge_warp) write_halo_mixed<EDF, S>(D, x, y, fout, smf + tid, ok, nf, uxf, uyf, gf, st, kImages);
+    if (edge_warp) write_halo_mixed<EDF, S>(D, x, y, fout, col, ok, nf, uxf, uyf, gf, st, kImages);
   return st;
+}
+
+// Momentum weights (p_s, p_s^2) of the shells in work units.
+struct PullW {
+  f2 p[6];
+};
+template <int EDF, class S>
+__device__ __forceinline__ PullW pull_weights(const DomDev& D) {
+  PullW w;
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    w.p[s] = f2_make(c_mt.p[EDF][s].x, c_mt.p[EDF][s].y);
+    if constexpr (S::kScaled) w.p[s] = vmul(w.p[s], f2_dup(D.a_s[s]));
+  }
+  return w;
+}
+// (A_d, B_d) of a direction from its three pairs in work units, shell after shell
+__device__ __forceinline__ f2 direction_sums(const f2 v[3], const PullW& w) {
+  f2 ab = vmul(f2_dup(f2_lo(v[0])), w.p[0]);
+  ab = vfma(f2_dup(f2_hi(v[0])), w.p[1], ab);
+#pragma unroll
+  for (int j = 1; j < 3; ++j) {
+    ab = vfma(f2_dup(f2_lo(v[j])), w.p[2 * j], ab);
+    ab = vfma(f2_dup(f2_hi(v[j])), w.p[2 * j + 1], ab);
+  }
+  return ab;
 }
 
 // Ask L2 for a tile's own blocks in rows y0-1 .. y0+kTileH of every plane: one
@@ -657,37 +847,38 @@ __device__ __forceinline__ void step_tile_mixed(const StepArgs& a, int t, float*
 #endif
   const long long c = cell_rel(D, x, y);
   const Nbr nb = neighbours(D, x, y);
-  // pull (FP32, deviation form) with the FP32 deviation moment sums
-  float A[12], B[12], pc[6], p2c[6];
-#pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    pc[s] = c_pf[EDF][s];
-    p2c[s] = c_p2f[EDF][s];
-  }
-#define RLBM_PULL_DIR(d)                                                        \
-  {                                                                             \
-    float a_ = 0.0f, b_ = 0.0f;                                                 \
-    _Pragma("unroll") for (int s = 0; s < 6; ++s) {                             \
-      const float v = S::decf(pull_one<d, float, S>(fin + c + (6 * d + s) * kBlkW, nb), D, s); \
-      smf[(6 * d + s) * kThreads + tid] = v;                                    \
-      a_ = fmaf(v, pc[s], a_);                                                  \
-      b_ = fmaf(v, p2c[s], b_);                                                 \
-    }                                                                           \
-    A[d] = a_;                                                                  \
-    B[d] = b_;                                                                  \
+  // pull (FP32, work units) with the FP32 deviation moment sums
+  f2 AB[12];
+  f2* col = reinterpret_cast<f2*>(smf) + tid;
+  const PullW w = pull_weights<EDF, S>(D);
+#define RLBM_PULL_DIR(d)                                                                       \
+  {                                                                                            \
+    f2 v_[3];                                                                                  \
+    _Pragma("unroll") for (int j = 0; j < 3; ++j) {                                            \
+      v_[j] = S::work2(pull_pair<d, PullF32, S>(fin + c + (3 * d + j) * kSegW, nb), D, 2 * j); \
+      col[(3 * d + j) * kThreads] = v_[j];                                                     \
+    }                                                                                          \
+    AB[d] = direction_sums(v_, w);                                                             \
   }
   RLBM_PULL_DIR(0) RLBM_PULL_DIR(1) RLBM_PULL_DIR(2) RLBM_PULL_DIR(3)
   RLBM_PULL_DIR(4) RLBM_PULL_DIR(5) RLBM_PULL_DIR(6) RLBM_PULL_DIR(7)
   RLBM_PULL_DIR(8) RLBM_PULL_DIR(9) RLBM_PULL_DIR(10) RLBM_PULL_DIR(11)
 #undef RLBM_PULL_DIR
-  const unsigned st = collide_mixed<EDF, S, false, kHalo>(D, x, y, c, A, B, smf, tid, fout);
+  const unsigned st = collide_mixed<EDF, S, false, kHalo>(D, x, y, c, AB, col, fout);
   if (st) atomicOr(a.status, st);
 }
 
 // kHalo = StepArgs::halo (see collide_mixed): 0 no halo writer, 0 and 1 no copy
 // of the relaxed values into the column.
+//
+// Bound: HBM for the FP32 storages (2048^2 periodic, FP32 deviations: 378 us, 6.39
+// TB/s of algorithmic traffic, 0.94 of the copy rate), instructions and load latency
+// for the 16-bit ones (332 us, 0.54 of it). Planes in pairs: one load or store moves
+// the shells s, s + 1 of a direction, and the pull, the sums and the synthesis work on
+// them as f32x2. With one plane per segment and scalar arithmetic the same step
+// issued about twice the instructions: 461 us (FP32 deviations), 500 us (BF16).
 template <int EDF, class S, int kHalo>
-__global__ void __launch_bounds__(kThreads, RLBM_MIXED_MIN_BLOCKS) k_step_mixed(StepArgs a) {
+__global__ void __launch_bounds__(kThreads, (mixed_min_blocks<S, kHalo>())) k_step_mixed(StepArgs a) {
   extern __shared__ float smf[];
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
@@ -696,10 +887,10 @@ __global__ void __launch_bounds__(kThreads, RLBM_MIXED_MIN_BLOCKS) k_step_mixed(
 }
 
 // ------------------------------------------- TMA-staged variant of the step
-// Per 32 x 4 tile and direction d, one TMA box brings the six shell planes of d
+// Per 32 x 4 tile and direction d, one TMA box brings the three plane pairs of d
 // for the tile's block of 32 cells and the blocks either side, rows y0-1 ..
-// y0+kTileH, into shared memory (a box {32 lanes, 6 planes, 3 blocks, kTileH + 2 rows} of the
-// 4D tensor {32, 72, nblk, ny + 2}); the bilinear pull reads its four
+// y0+kTileH, into shared memory (a box {64 elements, 3 pairs, 3 blocks, kTileH + 2 rows} of the
+// 4D tensor {64, 36, nblk, ny + 2}); the bilinear pull reads its four
 // neighbours there at fixed offsets (x - 1 of lane 0 and x + 1 of lane 31 in
 // the neighbouring blocks). A ring of kStages boxes keeps the next directions --
 // and, while a tile collides, the next tile's first directions -- in flight.
@@ -708,8 +899,7 @@ __global__ void __launch_bounds__(kThreads, RLBM_MIXED_MIN_BLOCKS) k_step_mixed(
 template <class S>
 struct TmaBox {
   using T = typename S::T;
-  static constexpr int kPlane = kBlkW;                        // a plane's 32 lanes
-  static constexpr int kBlock = kBoxPlanes * kPlane;          // six planes of one block
+  static constexpr int kBlock = kBoxPairs * kSegW;            // three pairs of one block
   static constexpr int kRow = kBoxBlocks * kBlock;            // three blocks of one row
   static constexpr unsigned kBytes = (unsigned)(kBoxElems * sizeof(T));
   static constexpr int kStageElems = kBoxElems;
@@ -728,50 +918,34 @@ __device__ __forceinline__ void tma_issue(const StepArgs& a, int t, int d, unsig
   const void* map = static_cast<const unsigned char*>(a.tmaps) + (size_t)tl.dom * kTensorMapBytes;
   const int k = d % kStages;
   mbar_expect_tx(&bar[k], TmaBox<S>::kBytes);
-  // lanes from 0, planes from 6d, blocks from the one left of the tile's
+  // elements from 0, pairs from 3d, blocks from the one left of the tile's
   // (x0 / 32 + 1 holds x0), rows from y = y0 - 1 (row index y0)
-  tma_load_4d(ring + k * TmaBox<S>::kBytes, map, 0, 6 * d, tl.x0 / kBlkW, tl.y0, &bar[k]);
+  tma_load_4d(ring + k * TmaBox<S>::kBytes, map, 0, 3 * d, tl.x0 / kBlkW, tl.y0, &bar[k]);
 }
 
 // Pull of direction d from its staged box; `cell` points at the cell's own
 // value in shell 0 of that stage, oxm / oxp are the offsets of x - 1 / x + 1
-// there (same weights and order of operations as pull_one), col at the
+// there (same weights and order of operations as pull_pair), col at the
 // thread's shared-memory column.
 template <int d, class S>
-__device__ __forceinline__ void pull_dir_staged(const typename S::T* cell, int oxm, int oxp, const DomDev& D,
-                                                const float pc[6], const float p2c[6], float* col, float& A,
-                                                float& B) {
-  using TB = TmaBox<S>;
-  constexpr double cx = dcos(d), cy = dsin(d);
-  constexpr int sx = sgnd(cx), sy = sgnd(cy);
-  constexpr double ax = dabs(cx), ay = dabs(cy);
-  constexpr float axr = (float)ax, ayr = (float)ay;
-  constexpr float w1 = axr * ayr, w2 = (1.0f - axr) * ayr, w3 = axr * (1.0f - ayr),
-                  w4 = (1.0f - axr) * (1.0f - ayr);
-  const int ox = sx > 0 ? oxm : (sx < 0 ? oxp : 0);
-  constexpr int oy = -sy * TB::kRow;
-  float a_ = 0.0f, b_ = 0.0f;
+__device__ __forceinline__ f2 pull_dir_staged(const typename S::T* cell, int oxm, int oxp, const DomDev& D,
+                                              const PullW& w, f2* col) {
+  Nbr nb;
+  nb.xm = oxm;
+  nb.xp = oxp;
+  nb.ym = -TmaBox<S>::kRow;
+  nb.yp = TmaBox<S>::kRow;
+  f2 v[3];
 #pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    const typename S::T* pl = cell + s * TB::kPlane;
-    float v;
-    if (ax == 0.0 || ay == 0.0) {
-      v = S::raw(pl[ox + oy]);
-    } else {
-      const float v1 = S::raw(pl[ox + oy]), v2 = S::raw(pl[oy]), v3 = S::raw(pl[ox]), v4 = S::raw(pl[0]);
-      v = fmaf(w1, v1, fmaf(w2, v2, fmaf(w3, v3, w4 * v4)));
-    }
-    v = S::decf(v, D, s);
-    col[(6 * d + s) * kThreads] = v;
-    a_ = fmaf(v, pc[s], a_);
-    b_ = fmaf(v, p2c[s], b_);
+  for (int j = 0; j < 3; ++j) {
+    v[j] = S::work2(pull_pair<d, PullF32, S>(cell + j * kSegW, nb), D, 2 * j);
+    col[(3 * d + j) * kThreads] = v[j];
   }
-  A = a_;
-  B = b_;
+  return direction_sums(v, w);
 }
 
 template <int EDF, class S>
-__global__ void __launch_bounds__(kThreads, RLBM_MIXED_MIN_BLOCKS) k_step_mixed_tma(StepArgs a) {
+__global__ void __launch_bounds__(kThreads, 512 / kThreads) k_step_mixed_tma(StepArgs a) {
   using T = typename S::T;
   using TB = TmaBox<S>;
   extern __shared__ __align__(128) unsigned char smt[];
@@ -799,16 +973,10 @@ __global__ void __launch_bounds__(kThreads, RLBM_MIXED_MIN_BLOCKS) k_step_mixed_
   }
   // the cell's own value in shell 0 of stage 0 (row ty + 1, middle block, lane
   // tx), the offsets of its x neighbours, and its column
-  const T* cell0 = reinterpret_cast<const T*>(ring) + (threadIdx.y + 1) * TB::kRow + TB::kBlock + threadIdx.x;
-  const int oxm = threadIdx.x > 0 ? -1 : -TB::kBlock + (kBlkW - 1);
-  const int oxp = threadIdx.x < kBlkW - 1 ? 1 : TB::kBlock - (kBlkW - 1);
-  float* col = smf + tid;
-  float pc[6], p2c[6];
-#pragma unroll
-  for (int s = 0; s < 6; ++s) {
-    pc[s] = c_pf[EDF][s];
-    p2c[s] = c_p2f[EDF][s];
-  }
+  const T* cell0 = reinterpret_cast<const T*>(ring) + (threadIdx.y + 1) * TB::kRow + TB::kBlock + 2 * threadIdx.x;
+  const int oxm = threadIdx.x > 0 ? -2 : -TB::kBlock + 2 * (kBlkW - 1);
+  const int oxp = threadIdx.x < kBlkW - 1 ? 2 : TB::kBlock - 2 * (kBlkW - 1);
+  f2* col = reinterpret_cast<f2*>(smf) + tid;
   unsigned it = 0;  // tiles done by this block: stage uses so far = it * 12 / kStages + d / kStages
   for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++it) {
     const Tile tl = a.tiles[t];
@@ -816,14 +984,15 @@ __global__ void __launch_bounds__(kThreads, RLBM_MIXED_MIN_BLOCKS) k_step_mixed_
     const int x = tl.x0 + threadIdx.x, y = tl.y0 + threadIdx.y;
     const int tnext = t + gridDim.x;
     const unsigned use0 = it * (12 / kStages);
-    float A[12], B[12];
+    const PullW w = pull_weights<EDF, S>(D);
+    f2 AB[12];
     // every lane pulls (lanes outside the domain read the box's padding and
     // fill only their own column, which is never stored)
 #define RLBM_STAGED_DIR(d)                                                                      \
   {                                                                                             \
     constexpr int k_ = (d) % kStages;                                                           \
     const bool ok_ = mbar_wait(&bar[k_], (use0 + (d) / kStages) & 1, wait_ns);                  \
-    pull_dir_staged<d, S>(cell0 + k_ * TB::kStageElems, oxm, oxp, D, pc, p2c, col, A[d], B[d]); \
+    AB[d] = pull_dir_staged<d, S>(cell0 + k_ * TB::kStageElems, oxm, oxp, D, w, col);           \
     if (__syncthreads_or(!ok_)) goto timed_out;                                                 \
     if (tid == 0) {                                                                             \
       inflight &= ~(1u << k_);                                                                  \
@@ -841,7 +1010,7 @@ __global__ void __launch_bounds__(kThreads, RLBM_MIXED_MIN_BLOCKS) k_step_mixed_
 #undef RLBM_STAGED_DIR
     if (x < D.nx && y < D.ny) {
       T* __restrict__ fout = static_cast<T*>(a.fout) + D.off;
-      const unsigned st = collide_mixed<EDF, S, true>(D, x, y, cell_rel(D, x, y), A, B, smf, tid, fout);
+      const unsigned st = collide_mixed<EDF, S, true>(D, x, y, cell_rel(D, x, y), AB, col, fout);
       if (st) atomicOr(a.status, st);
     }
   }
@@ -871,66 +1040,44 @@ __global__ void __launch_bounds__(kThreads) k_fields_mixed(FieldsArgs a) {
   if (x >= D.nx || y >= D.ny) return;
   const typename S::T* __restrict__ f = static_cast<const typename S::T*>(a.f) + D.off;
   const long long c = cell_rel(D, x, y);
-  float A[12], B[12];
+  f2 AB[12];
   {
-    float pc[6], p2c[6];
-#pragma unroll
-    for (int s = 0; s < 6; ++s) {
-      pc[s] = c_pf[EDF][s];
-      p2c[s] = c_p2f[EDF][s];
-    }
+    const PullW w = pull_weights<EDF, S>(D);
     const Nbr nb = neighbours(D, x, y);
     const bool streamed = a.streamed != 0;
-#define RLBM_FIELDS_DIR(d)                                                                       \
-  {                                                                                              \
-    float a_ = 0.0f, b_ = 0.0f;                                                                  \
-    _Pragma("unroll") for (int s = 0; s < 6; ++s) {                                              \
-      const typename S::T* pl = f + c + (6 * d + s) * kBlkW;                                     \
-      const float r = streamed ? pull_one<d, float, S>(pl, nb) : S::raw(pl[0]);                  \
-      const float v = S::decf(r, D, s);                                                          \
-      a_ = fmaf(v, pc[s], a_);                                                                   \
-      b_ = fmaf(v, p2c[s], b_);                                                                  \
-    }                                                                                            \
-    A[d] = a_;                                                                                   \
-    B[d] = b_;                                                                                   \
+#define RLBM_FIELDS_DIR(d)                                                                          \
+  {                                                                                                 \
+    f2 v_[3];                                                                                       \
+    _Pragma("unroll") for (int j = 0; j < 3; ++j) {                                                 \
+      const typename S::T* pl = f + c + (3 * d + j) * kSegW;                                        \
+      const f2 r = streamed ? pull_pair<d, PullF32, S>(pl, nb)                                      \
+                            : S::raw2(*reinterpret_cast<const Pair<typename S::T>*>(pl));           \
+      v_[j] = S::work2(r, D, 2 * j);                                                                \
+    }                                                                                               \
+    AB[d] = direction_sums(v_, w);                                                                  \
   }
     RLBM_FIELDS_DIR(0) RLBM_FIELDS_DIR(1) RLBM_FIELDS_DIR(2) RLBM_FIELDS_DIR(3)
     RLBM_FIELDS_DIR(4) RLBM_FIELDS_DIR(5) RLBM_FIELDS_DIR(6) RLBM_FIELDS_DIR(7)
     RLBM_FIELDS_DIR(8) RLBM_FIELDS_DIR(9) RLBM_FIELDS_DIR(10) RLBM_FIELDS_DIR(11)
 #undef RLBM_FIELDS_DIR
   }
-  const HarmF ha = harmonics_f(A), hb = harmonics_f(B);
-  const df N0 = df_add(df_make(D.n0_hl[0], D.n0_hl[1]), ha.h0);
-  const df H0 = df_add(df_make(D.t00_hl[0], D.t00_hl[1]), hb.h0);
-  df T[6];
-  T[0] = H0;
-  T[1] = df_make(hb.c1, 0.0f);
-  T[2] = df_make(hb.s1, 0.0f);
-  T[3] = df_scale(df_add(H0, hb.c2), 0.5f);
-  T[4] = df_make(0.5f * hb.s2, 0.0f);
-  T[5] = df_scale(df_add(H0, -hb.c2), 0.5f);
-  df ux, uy, eps, gam;
-  unsigned st = landau_df(T, ux, uy, eps, gam);
-  df n = df_make(0.0f, 0.0f);
-  if (!(st & ST_NONPHYSICAL)) {
-    n = df_mul(gam, df_sub(N0, df_add(df_mul(ux, ha.c1), df_mul(uy, ha.s1))));
-    if (!(n.hi > 0.0f) || !isfinite(n.hi)) st |= ST_NONPHYSICAL;
-  }
+  FrameDf F;
+  unsigned st = landau_df(moments_df(D, AB), F);
   double on = nan(""), oth = nan(""), oux = nan(""), ouy = nan(""), oz = nan("");
   if (!(st & ST_NONPHYSICAL)) {
-    const float nf = df_to_float(n), ef = df_to_float(eps);
+    const float nf = df_to_float(F.n), ef = df_to_float(F.eps);
     float theta, z, g[6];
     if (EDF == EDF_MJ) {
       theta = ef / (2.0f * nf);
       z = nf / (2.0f * kPIf * theta * theta);
     } else {
-      const float target = 0.5f * kPIf * ef * ef / (nf * nf * nf);
-      const int zs = solve_z_R_f<EDF>(target, z, g);
+      const int zs = solve_z_R_f<EDF, S::kScaled, true>(nf, ef, z, g);
       st |= zs;
       if (zs & ST_CLAMPED) theta = sqrtf(nf / (2.0f * kPIf * g[1]));
       else theta = 0.5f * g[1] / g[2] * ef / nf;
     }
-    on = (double)n.hi + (double)n.lo;
+    const df ux = df_first(F.u), uy = df_second(F.u);
+    on = (double)F.n.hi + (double)F.n.lo;
     oux = (double)ux.hi + (double)ux.lo;
     ouy = (double)uy.hi + (double)uy.lo;
     oth = theta;
@@ -982,48 +1129,34 @@ __global__ void __launch_bounds__(kThreads) k_init_mixed(InitArgs a) {
     n = 2.0f * kPIf * theta * theta * g[1];
   } else {
     n = (float)a.a[i];
-    st |= (theta > 0.0f && n > 0.0f) ? solve_z_nt_f<EDF>(n, theta, z, g) : 0;
+    st |= (theta > 0.0f && n > 0.0f) ? solve_z_nt_f<EDF, S::kScaled, true>(n, theta, z, g) : 0;
   }
-  const float u2 = ux * ux + uy * uy;
+  const float u2 = fmaf(ux, ux, __fmul_rn(uy, uy));
   const bool ok = (u2 < 1.0f) && (theta > 0.0f) && (n > 0.0f) && isfinite(z) && isfinite(u2);
   if (!ok) st |= ST_NONPHYSICAL;
   const float gam = ok ? 1.0f / sqrtf(1.0f - u2) : 1.0f;
   typename S::T* __restrict__ f = static_cast<typename S::T*>(a.f) + D.off;
   const long long c = cell_rel(D, x, y);
-  float* col = smi + tid;
+  f2* col = reinterpret_cast<f2*>(smi) + tid;
+  using P = Pair<typename S::T>;
   if (ok) {
-    float zr[21], zi[21];
-    dz_moments<EDF>(D, g, theta, ux, uy, gam, -1.0f, -1.0f, zr, zi);
-    float d10 = 0.0f, d20 = 0.0f, d21r = 0.0f, d21i = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      d10 = fmaf(c_Ef[EDF][k], zr[k * (k + 1) / 2], d10);
-      d20 = fmaf(c_Ef[EDF][6 + k], zr[k * (k + 1) / 2], d20);
-    }
-#pragma unroll
-    for (int k = 1; k < 6; ++k) {
-      d21r = fmaf(c_Ef[EDF][12 + k], zr[k * (k + 1) / 2 + 1], d21r);
-      d21i = fmaf(c_Ef[EDF][12 + k], zi[k * (k + 1) / 2 + 1], d21i);
-    }
-    zr[1] -= d10;
-    zr[3] -= d20;
-    zr[4] -= d21r;
-    zi[4] -= d21i;
+    EqF q;
+    dz_moments<EDF>(D, g, theta, ux, uy, gam, -1.0f, -1.0f, q);
+    remove_defects<EDF>(q);
 #pragma unroll 1
-    for (int s = 0; s < 6; ++s) {
-      float fe[12];
-      dfeq_shell<EDF>(s, D.rres[s], zr, zi, fe);
+    for (int j = 0; j < 3; ++j) {
+      f2 fe[12];
+      dfeq_work<EDF, S>(D, j, q, fe);
 #pragma unroll
       for (int d = 0; d < 12; ++d) {
-        const int q = 6 * d + s;
-        col[q * kThreads] = fe[d];
-        f[q * kBlkW + c] = S::encf(fe[d], D, s);
+        col[(3 * d + j) * kThreads] = fe[d];
+        *reinterpret_cast<P*>(f + c + (3 * d + j) * kSegW) = S::enc2(fe[d], D, 2 * j);
       }
     }
   } else {
-    for (int q = 0; q < 72; ++q) {
-      col[q * kThreads] = __int_as_float(0x7fc00000);  // NaN
-      f[q * kBlkW + c] = S::encf(col[q * kThreads], D, q % 6);
+    for (int k = 0; k < kPairs; ++k) {
+      col[k * kThreads] = f2_dup(__int_as_float(0x7fc00000));  // NaN
+      *reinterpret_cast<P*>(f + c + k * kSegW) = S::enc2(col[k * kThreads], D, 2 * (k % 3));
     }
   }
   write_halo_mixed<EDF, S>(D, x, y, f, col, ok, n, ux, uy, gam, st, true);
@@ -1072,8 +1205,8 @@ __global__ void k_prepare_refs(DomDev* doms, int ndom) {
   D.t00ref = t00;
   double r1 = 0.0, r2 = 0.0;
   for (int s = 0; s < 6; ++s) {
-    r1 += 12.0 * (double)D.rres[s] * (double)c_pf[EDF][s];
-    r2 += 12.0 * (double)D.rres[s] * (double)c_p2f[EDF][s];
+    r1 += 12.0 * (double)D.rres[s] * (double)c_mt.p[EDF][s].x;
+    r2 += 12.0 * (double)D.rres[s] * (double)c_mt.p[EDF][s].y;
   }
   D.zeff1 = n0 + r1;
   D.zeff2 = t00 + r2;
@@ -1087,15 +1220,6 @@ __global__ void k_prepare_refs(DomDev* doms, int ndom) {
 }
 
 // ------------------------------------------------------------- launchers
-static const double h_p2[3][6] = {RLBM_P2_MJ_INIT, RLBM_P2_FD_INIT, RLBM_P2_BE_INIT};
-static const double h_pnk[63] = RLBM_PNK_INIT;
-static const double h_invpow[6 * RLBM_NSERIES] = RLBM_INVPOW_INIT;
-static const double h_be_exp[6 * RLBM_NEXP] = RLBM_BE_EXP_INIT;
-static const double h_fd_exp[6 * RLBM_NEXP] = RLBM_FD_EXP_INIT;
-static const double h_be_logcoef[6] = RLBM_BE_LOGCOEF_INIT;
-static const double h_be_harm[6] = RLBM_BE_HARM_INIT;
-static const double h_g_zc[6] = RLBM_G_ZC_INIT;
-
 template <class S, int EDF>
 static cudaError_t prepare_tma_t() {
   cudaError_t e = cudaFuncSetAttribute(k_step_mixed_tma<EDF, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1129,33 +1253,6 @@ static cudaError_t prepare_s() {
   if ((e = prepare_common_t<S, EDF_FD>())) return e;
   return prepare_common_t<S, EDF_BE>();
 }
-
-// Upload the FP32 tables of this translation unit (converted once from the FP64
-// tables).
-static cudaError_t upload_mixed_tables() {
-  float p2f[3][6], pnk[63], inv[6 * kSerF], be[6 * kExpBEf], fd[6 * kExpFDf], lc[6], hm[6], gz[6];
-  for (int e = 0; e < 3; ++e)
-    for (int s = 0; s < 6; ++s) p2f[e][s] = (float)h_p2[e][s];
-  for (int i = 0; i < 63; ++i) pnk[i] = (float)h_pnk[i];
-  for (int nu = 0; nu < 6; ++nu) {
-    for (int k = 0; k < kSerF; ++k) inv[nu * kSerF + k] = (float)h_invpow[nu * RLBM_NSERIES + k];
-    for (int k = 0; k < kExpBEf; ++k) be[nu * kExpBEf + k] = (float)h_be_exp[nu * RLBM_NEXP + k];
-    for (int k = 0; k < kExpFDf; ++k) fd[nu * kExpFDf + k] = (float)h_fd_exp[nu * RLBM_NEXP + k];
-    lc[nu] = (float)h_be_logcoef[nu];
-    hm[nu] = (float)h_be_harm[nu];
-    gz[nu] = (float)h_g_zc[nu];
-  }
-  cudaError_t e;
-  if ((e = cudaMemcpyToSymbol(c_p2f, p2f, sizeof(p2f)))) return e;
-  if ((e = cudaMemcpyToSymbol(c_pnkf, pnk, sizeof(pnk)))) return e;
-  if ((e = cudaMemcpyToSymbol(c_invpowf, inv, sizeof(inv)))) return e;
-  if ((e = cudaMemcpyToSymbol(c_be_expf, be, sizeof(be)))) return e;
-  if ((e = cudaMemcpyToSymbol(c_fd_expf, fd, sizeof(fd)))) return e;
-  if ((e = cudaMemcpyToSymbol(c_be_logcoeff, lc, sizeof(lc)))) return e;
-  if ((e = cudaMemcpyToSymbol(c_be_harmf, hm, sizeof(hm)))) return e;
-  return cudaMemcpyToSymbol(c_g_zcf, gz, sizeof(gz));
-}
-
 
 template <class S>
 static cudaError_t step_s(int edf, const StepArgs& a, int grid, cudaStream_t s) {
@@ -1195,11 +1292,10 @@ struct MixedUnit {
   cudaError_t (*copy)(const CopyArgs& a, cudaStream_t s);
 };
 
-// Tables of this unit, shared-memory limits of its kernels.
+// Shared-memory limits of this unit's kernels.
 template <class S>
 static cudaError_t prepare_unit() {
-  cudaError_t e = upload_mixed_tables();
-  return e != cudaSuccess ? e : prepare_s<S>();
+  return prepare_s<S>();
 }
 
 template <class S>

@@ -40,7 +40,7 @@ EDFS = ("MJ", "FD", "BE")
 NSERIES = 64       # power-series terms tabulated (k = 1..NSERIES)
 NEXP = 48          # mu-expansion terms tabulated
 NLOGSER = 30       # terms of the series in u = -ln(1 - x)
-NREV = 10          # terms of the reversion t(w)
+NREV = 10          # terms of the reversions t(w), t(G)
 
 
 def moments(edf):
@@ -164,9 +164,10 @@ def log_series_tables():
     """Series of the polylogs in u = -ln(1 - x): Li_nu(x) = sum_n c_nu[n] u^(n+1), from
     Li_1 = u and dLi_nu/du = Li_(nu-1) / (e^u - 1), in exact rational arithmetic
     (convergence radius 2 pi, so a few terms cover what takes dozens in x), nu = 2..6;
-    and, with g_nu = s Li_nu(s z), t = g_1 = s u (s = -1 FD, +1 BE): the reversion
-    t = w sum_n a_n w^n of w = g_2^3 / g_3^2 = t - (47/1728) t^3 - ..., s = +1 (for
-    s = -1 the a_n of odd n change sign)."""
+    and, with g_nu = s Li_nu(s z), t = g_1 = s u (s = -1 FD, +1 BE): the reversions
+    t = w sum_n a_n w^n of w = g_2^3 / g_3^2 = t - (47/1728) t^3 - ... and
+    t = G sum_n b_n G^n of G = g_2 = t - t^2/4 + ..., both for s = +1 (for s = -1
+    the coefficients of odd n change sign)."""
     from fractions import Fraction as Fr
     from math import factorial
     N = NLOGSER
@@ -187,14 +188,18 @@ def log_series_tables():
     W = [Fr(0)]
     for k in range(M - 1):  # w / t
         W.append((num[k] - sum(W[j + 1] * den[k - j] for j in range(k))) / den[0])
-    t = [Fr(0), Fr(1)] + [Fr(0)] * (M - 2)
-    for _ in range(M):
-        comp, pw = [Fr(0)] * M, [Fr(1)] + [Fr(0)] * (M - 1)
-        for k in range(M):
-            comp = [c + W[k] * p for c, p in zip(comp, pw)]
-            pw = mul(pw, t, M)
-        t = [x - (c - int(i == 1)) for i, (x, c) in enumerate(zip(t, comp))]
-    return [[float(c) for c in S[nu]] for nu in range(2, 7)], [float(c) for c in t[1:]]
+
+    def revert(W):
+        t = [Fr(0), Fr(1)] + [Fr(0)] * (M - 2)
+        for _ in range(M):
+            comp, pw = [Fr(0)] * M, [Fr(1)] + [Fr(0)] * (M - 1)
+            for k in range(M):
+                comp = [c + W[k] * p for c, p in zip(comp, pw)]
+                pw = mul(pw, t, M)
+            t = [x - (c - int(i == 1)) for i, (x, c) in enumerate(zip(t, comp))]
+        return [float(c) for c in t[1:]]
+
+    return [[float(c) for c in S[nu]] for nu in range(2, 7)], revert(W), revert([Fr(0)] + S[2][:M - 1])
 
 
 def c_arr(name, vals, ctype="double", per_line=4):
@@ -254,10 +259,11 @@ def main():
     hdr.append(c_arr("RLBM_BE_LOGCOEF", rfact))
     hdr.append(c_arr("RLBM_BE_HARM", harm))
     hdr.append(c_arr("RLBM_G_ZC", gzc))
-    logser, rev = log_series_tables()
+    logser, rev, revg = log_series_tables()
     hdr.append("#define RLBM_NLOGSER %d\n#define RLBM_NREV %d" % (NLOGSER, NREV))
     hdr.append(c_arr("RLBM_LOGSER", [x for row in logser for x in row]))
     hdr.append(c_arr("RLBM_REV", rev))
+    hdr.append(c_arr("RLBM_REVG", revg))
     rzc = mp.polylog(3, ZC) ** 2 / mp.polylog(2, ZC) ** 3
     hdr.append("#define RLBM_R_ZC %r\n" % float(rzc))
     hdr.append("#endif")
