@@ -18,6 +18,12 @@ using namespace rlbm;
 namespace {
 
 constexpr size_t kAlign = 256;
+// A mixed launch of at most this many tiles is one wave (4 blocks on each of 152 SMs) and
+// lasts as long as its longest block. There the packed tiles go one warp to a block
+// (kOneWarp): a packed warp's accesses touch up to 32 rows, so four in one SM were the
+// pole (129^2 domain: 17.4 us a step, 128^2: 5.6 us). Larger launches keep whole
+// tiles, whose fourth of the blocks matters more.
+constexpr size_t kOneWaveTiles = 4 * 152;
 constexpr int kChunkPairs = 16;  // a chunk graph holds 2 * kChunkPairs steps
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -38,8 +44,11 @@ struct Layout {
   size_t status_off = 0, doms_off = 0, tiles_off = 0, ptiles_off = 0, tmaps_off = 0, pop_off[2] = {0, 0};
   size_t pop_elems = 0, pop_bytes = 0, total = 0;
   std::vector<DomDev> dd;
-  std::vector<Tile> tiles;   // kTileW x kTileH tiles: every kernel but the mixed L1 step
+  std::vector<Tile> tiles;   // kTileW x kTileH tiles: the TMA-staged step, initialisers, read-outs
   std::vector<Tile> ptiles;  // the same with each domain's ragged last x block packed (Tile::w)
+  std::vector<Tile> otiles;  // that at one warp per packed tile (see kOneWaveTiles), or empty
+  // what the FP64 and the mixed L1 step walk
+  const std::vector<Tile>& stiles() const { return otiles.empty() ? ptiles : otiles; }
 };
 
 bool valid_bc(int b) {
@@ -134,6 +143,15 @@ void make_layout(const rlbm_config* c, Layout& L) {
       }
     }
   }
+  L.otiles.clear();
+  if (c->storage != RLBM_F64 && L.ptiles.size() <= kOneWaveTiles)
+    for (const Tile& t : L.ptiles) {
+      const int r = packed_rows_per_warp(t.w);
+      if (!t.w) L.otiles.push_back(t);
+      else
+        for (int k = 0; k < kTileH && t.y0 + k * r < L.dd[t.dom].ny; ++k)
+          L.otiles.push_back(Tile{t.dom, t.x0, t.y0 + k * r, t.w + kOneWarp});
+    }
   L.pop_elems = off;
   L.pop_bytes = align_up(off * es, kAlign);
   size_t b = 0;
@@ -144,7 +162,7 @@ void make_layout(const rlbm_config* c, Layout& L) {
   L.tiles_off = b;
   b = align_up(b + sizeof(Tile) * L.tiles.size(), kAlign);
   L.ptiles_off = b;
-  b = align_up(b + sizeof(Tile) * L.ptiles.size(), kAlign);
+  b = align_up(b + sizeof(Tile) * L.stiles().size(), kAlign);
   // TMA descriptors of the staged mixed step: [copy][domain]
   L.tmaps_off = b;
   if (c->storage != RLBM_F64) b = align_up(b + 2 * (size_t)kTensorMapBytes * L.dd.size(), kAlign);
@@ -189,17 +207,18 @@ namespace {
 
 int cuda_fail(cudaError_t e) { return e == cudaSuccess ? RLBM_OK : RLBM_E_CUDA; }
 
-// The tile list a step launch walks: the packed one for the mixed step's L1
-// pull, the plain one for the TMA-staged variant (whose boxes assume 32 x
-// kTileH tiles) and the FP64 step.
-bool packed_tiles(const rlbm_ctx* h) { return h->storage != RLBM_F64 && h->kernel == RLBM_KERNEL_L1; }
+// The tile list a step launch walks: the packed one for the FP64 step (3 % on the
+// 256-domain batch: an FP64 instruction takes as long with idle lanes) and the mixed
+// step's L1 pull, the plain one for the TMA-staged variant (whose boxes assume 32 x
+// kTileH tiles). The steps on the packed list leave the periodic halo images unwritten.
+bool packed_tiles(const rlbm_ctx* h) { return h->kernel == RLBM_KERNEL_L1; }
 
 cudaError_t launch_step(rlbm_ctx* h, int from) {
   StepArgs a;
   a.doms = h->d_doms;
   const bool pk = packed_tiles(h);
   a.tiles = pk ? h->d_ptiles : h->d_tiles;
-  a.ntiles = (int)(pk ? h->L.ptiles.size() : h->L.tiles.size());
+  a.ntiles = (int)(pk ? h->L.stiles().size() : h->L.tiles.size());
   a.fin = h->pop[from];
   a.fout = h->pop[1 - from];
   a.status = h->d_status;
@@ -210,6 +229,7 @@ cudaError_t launch_step(rlbm_ctx* h, int from) {
   a.variant = h->kernel;
   a.wait_ns = h->wait_ns;
   a.halo = h->halo;
+  a.images = 0;
   const int grid = h->grid > 0 ? h->grid : a.ntiles;
   if (h->storage == RLBM_F64) return launch_step_f64(h->edf, a, grid, h->stream);
   return launch_step_mixed(h->storage, h->edf, a, grid, h->stream);
@@ -454,7 +474,7 @@ int rlbm_create(const rlbm_config* c, rlbm_handle* out) {
   for (const rlbm_domain& d : h->doms) {
     h->cells += (long long)d.nx * d.ny;
     for (int b : {d.bc_xlo, d.bc_xhi, d.bc_ylo, d.bc_yhi})
-      if (bc_writes_halo(b)) h->halo = std::max(h->halo, b == RLBM_FIXED_T_WALL ? 1 : 2);
+      if (bc_writes_halo(b)) h->halo = std::max(h->halo, b == RLBM_FIXED_T_WALL ? 1 : (b == RLBM_VELOCITY_WALL ? 3 : 2));
   }
   h->base = static_cast<char*>(c->device_buffer);
   h->d_status = reinterpret_cast<unsigned*>(h->base + h->L.status_off);
@@ -482,7 +502,7 @@ int rlbm_create(const rlbm_config* c, rlbm_handle* out) {
     e = cudaMemcpyAsync(h->d_tiles, h->L.tiles.data(), sizeof(Tile) * h->L.tiles.size(),
                         cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h->d_ptiles, h->L.ptiles.data(), sizeof(Tile) * h->L.ptiles.size(),
+    e = cudaMemcpyAsync(h->d_ptiles, h->L.stiles().data(), sizeof(Tile) * h->L.stiles().size(),
                         cudaMemcpyHostToDevice, h->stream);
   std::vector<unsigned char> maps;
   if (e == cudaSuccess && h->d_tmaps && !encode_tmaps(h, maps)) h->d_tmaps = nullptr;
@@ -576,7 +596,7 @@ int rlbm_step(rlbm_handle h, int nsteps) {
     h->cur = 1 - h->cur;
     launches += 1;
   }
-  if (nsteps > 0 && packed_tiles(h)) h->images_stale = true;  // the L1 step wraps instead
+  if (nsteps > 0 && packed_tiles(h)) h->images_stale = true;  // those steps wrap instead
   h->last_updates = (long long)nsteps * h->cells;
   h->last_launches = launches;
   return cuda_fail(e);
@@ -774,6 +794,8 @@ int rlbm_get_populations(rlbm_handle h, int domain, double* f, int on_device) {
 }
 
 int rlbm_set_populations(rlbm_handle h, int domain, const double* f, int on_device) {
+  // (the images of the other domains first: filling them later would overwrite f's halo)
+  if (h && domain >= 0 && domain < h->ndom && f && fill_images(h) != cudaSuccess) return RLBM_E_CUDA;
   return copy_pops(h, domain, const_cast<double*>(f), on_device, 0);
 }
 
@@ -799,7 +821,7 @@ int rlbm_tune(rlbm_handle h, int repeats) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return RLBM_E_CUDA;
   // grid 0: one block per tile of whichever list the variant walks
-  const int ntiles = (int)h->L.ptiles.size();  // the shorter list
+  const int ntiles = (int)h->L.stiles().size();
   std::vector<int> cand = {0};
   for (int k : {1, 2, 3, 4, 6, 8})
     if (k * sms < ntiles) cand.push_back(k * sms);
@@ -843,7 +865,7 @@ int rlbm_tune(rlbm_handle h, int repeats) {
   cudaEventDestroy(t1);
   h->grid = best_grid;
   h->kernel = best_kernel;
-  if (best_grid == 0) best_grid = (int)(packed_tiles(h) ? h->L.ptiles.size() : h->L.tiles.size());
+  if (best_grid == 0) best_grid = (int)(packed_tiles(h) ? h->L.stiles().size() : h->L.tiles.size());
   drop_graphs(h);
   *h->h_status = saved;
   if (e == cudaSuccess)

@@ -90,10 +90,14 @@ constexpr int kTileW = 32, kTileH = RLBM_TILE_H;
 // block of a domain, only w cells wide, packed: each warp covers 32 / w rows of
 // w cells (lane l on x0 + l % w, row y0 + k * (32 / w) + l / w; lanes from
 // (32 / w) * w on idle), so the tile spans kTileH * (32 / w) rows.
+// With kOneWarp added to w only warp 0 of the tile works: a launch of one wave is as
+// long as its longest block, and the accesses of a packed warp take a sector per
+// row, so there each packed warp gets a block of its own (see make_layout).
 struct Tile {
   int dom, x0, y0, w;
 };
 constexpr int kPackMaxW = 16;  // widest ragged block worth packing (two rows per warp)
+constexpr int kOneWarp = 256;
 
 __host__ __device__ constexpr int packed_rows_per_warp(int w) { return w > 0 ? kTileW / w : 1; }
 
@@ -105,10 +109,10 @@ __host__ __device__ inline bool tile_cell(const Tile& tl, int lane, int warp, in
     y = tl.y0 + warp;
     return true;
   }
-  const int r = kTileW / tl.w;
-  x = tl.x0 + lane % tl.w;
-  y = tl.y0 + warp * r + lane / tl.w;
-  return lane < r * tl.w;
+  const int w = tl.w & (kOneWarp - 1), r = kTileW / w;
+  x = tl.x0 + lane % w;
+  y = tl.y0 + warp * r + lane / w;
+  return lane < r * w && (warp == 0 || tl.w < kOneWarp);
 }
 
 struct StepArgs {
@@ -121,7 +125,10 @@ struct StepArgs {
   const void* tmaps;      // TMA load descriptors of fin, one per domain (kTensorMapBytes each), or null
   int variant;            // mixed step kernel (RLBM_KERNEL_*); the FP64 step has one
   int halo;               // halo work of the launch: 0 none (every side periodic or exchanged),
-                          // 1 wall equilibria only, 2 also zero-gradient copies
+                          // 1 wall equilibria only, 2 also zero-gradient copies, 3 also velocity
+                          // walls (FP64 storage only)
+  int images;             // FP64 step: write the periodic halo images (callers that hand out the
+                          // halo as stored); the pull wraps and does not read them
   unsigned long long wait_ns;  // limit of the TMA variant's copy waits (0: kDefaultWaitNs)
 };
 

@@ -556,11 +556,10 @@ struct CellState {
   double g[6];
 };
 
-// kZ: z is wanted (the read-out; a step only needs the g_nu).
-template <int EDF, bool kZ>
-__device__ __forceinline__ int cell_state(const double N[3], const double T[6], CellState& S) {
+// The frame and n of a cell.
+__device__ __forceinline__ int cell_frame(const double N[3], const double T[6], CellState& S) {
   Frame F;
-  int st = landau(T, F);
+  const int st = landau(T, F);
   if (st & ST_NONPHYSICAL) return st;
   S.ux = F.ux;
   S.uy = F.uy;
@@ -568,6 +567,13 @@ __device__ __forceinline__ int cell_state(const double N[3], const double T[6], 
   S.eps = F.eps;
   S.n = F.gamma * fma(-F.ux, N[1], fma(-F.uy, N[2], N[0]));
   if (!(S.n > 0.0) || !isfinite(S.n) || !isfinite(S.eps)) return st | ST_NONPHYSICAL;
+  return st;
+}
+
+// theta and the g_nu from n and eps. kZ: z is wanted (the read-out; a step only needs
+// the g_nu).
+template <int EDF, bool kZ>
+__device__ __forceinline__ int cell_theta(CellState& S) {
   if (EDF == EDF_MJ) {
     S.theta = 0.5 * (S.eps * rcp64(S.n));
     if (kZ) {
@@ -575,14 +581,20 @@ __device__ __forceinline__ int cell_state(const double N[3], const double T[6], 
 #pragma unroll
       for (int i = 0; i < 6; ++i) S.g[i] = S.z;
     }
-    return st;
+    return 0;
   }
   const double rn = rcp64(S.n), en = S.eps * rn;
   const double target = (0.5 * PI) * (en * en * rn);
   const int zs = solve_z_from_R<EDF, kZ>(target, S.z, S.g);
-  st |= zs;
   if (zs & ST_CLAMPED) S.theta = sqrt(S.n / (2.0 * PI * S.g[1]));
   else S.theta = 0.5 * (S.g[1] * rcp64(S.g[2])) * en;
+  return zs;
+}
+
+template <int EDF, bool kZ>
+__device__ __forceinline__ int cell_state(const double N[3], const double T[6], CellState& S) {
+  int st = cell_frame(N, T, S);
+  if (!(st & ST_NONPHYSICAL)) st |= cell_theta<EDF, kZ>(S);
   return st;
 }
 
@@ -688,11 +700,9 @@ __device__ __forceinline__ DirPow dir_powers(double ux, double uy) {
 // Discrete equilibrium of one shell s at the 12 directions (order index oi =
 // N - 2; the fifth order by default):
 //   f^eq_{ds} = sum_k R_k C_k(d),  R_k = sum_{n>=k} Q^(k)_{s n} Y_nk,
-// even k the same and odd k of opposite sign at d + 6.
+// even k the same (E) and odd k of opposite sign (O) at d + 6.
 template <int EDF>
-__device__ __forceinline__ void feq_shell(int s, const double y[21], const DirPow& C, double fe[12],
-                                          int oi = kOrder5) {
-  double R[6];
+__device__ __forceinline__ void shell_project(int s, const double y[21], double R[6], int oi = kOrder5) {
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     double a = c_Q[oi][EDF][qoff(k) + s * (6 - k)] * y[k * (k + 1) / 2 + k];
@@ -700,14 +710,27 @@ __device__ __forceinline__ void feq_shell(int s, const double y[21], const DirPo
     for (int n = k + 1; n < 6; ++n) a = fma(c_Q[oi][EDF][qoff(k) + s * (6 - k) + (n - k)], y[n * (n + 1) / 2 + k], a);
     R[k] = a;
   }
+}
+
+// E and O of direction d < 6; p3 = R_3 Re w^3, q3 = R_3 Im w^3 (C_3(d): Re, Im, -Re,
+// -Im, Re, Im of w^3).
+__device__ __forceinline__ void synth_dir(int d, const double R[6], double p3, double q3, const DirPow& C, double& E,
+                                          double& O) {
+  const double o3 = d % 2 ? (d == 3 ? -q3 : q3) : (d == 2 ? -p3 : p3);
+  E = fma(d < 3 ? R[2] : -R[2], C.c2[d % 3], fma(R[4], C.c4[d % 3], R[0]));
+  O = fma(R[1], C.c1[d], fma(R[5], C.c5[d], o3));
+}
+
+template <int EDF>
+__device__ __forceinline__ void feq_shell(int s, const double y[21], const DirPow& C, double fe[12],
+                                          int oi = kOrder5) {
+  double R[6];
+  shell_project<EDF>(s, y, R, oi);
   const double p3 = R[3] * C.w3r, q3 = R[3] * C.w3i;
-  // C_3(d): Re, Im, -Re, -Im, Re, Im of w^3
-  const double o3[6] = {p3, q3, -p3, -q3, p3, q3};
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
-    const double t = fma(R[4], C.c4[d % 3], R[0]);
-    const double E = fma(d < 3 ? R[2] : -R[2], C.c2[d % 3], t);
-    const double O = fma(R[1], C.c1[d], fma(R[5], C.c5[d], o3[d]));
+    double E, O;
+    synth_dir(d, R, p3, q3, C, E, O);
     fe[d] = E + O;
     fe[d + 6] = E - O;
   }
@@ -720,13 +743,7 @@ struct Harm {
   double h0, c1, s1, c2, s2;
 };
 
-__device__ __forceinline__ Harm harmonics(const double v[12], bool need2) {
-  double e[6], o[6];
-#pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    e[d] = v[d] + v[d + 6];
-    o[d] = v[d] - v[d + 6];
-  }
+__device__ __forceinline__ Harm harmonics_eo(const double e[6], const double o[6], bool need2) {
   const double h = SQRT3_2;
   Harm H;
   H.h0 = ((e[0] + e[1]) + (e[2] + e[3])) + (e[4] + e[5]);
@@ -739,6 +756,25 @@ __device__ __forceinline__ Harm harmonics(const double v[12], bool need2) {
     H.c2 = H.s2 = 0.0;
   }
   return H;
+}
+
+__device__ __forceinline__ Harm harmonics(const double v[12], bool need2) {
+  double e[6], o[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    e[d] = v[d] + v[d + 6];
+    o[d] = v[d] - v[d + 6];
+  }
+  return harmonics_eo(e, o, need2);
+}
+
+// N^mu and T^{mu nu} from the harmonic sums of A_d and B_d.
+__device__ __forceinline__ void moments_of(const Harm& ha, const Harm& hb, double N[3], double T[6]) {
+  N[0] = ha.h0; N[1] = ha.c1; N[2] = ha.s1;
+  T[0] = hb.h0; T[1] = hb.c1; T[2] = hb.s1;
+  T[3] = 0.5 * (hb.h0 + hb.c2);
+  T[4] = 0.5 * hb.s2;
+  T[5] = 0.5 * (hb.h0 - hb.c2);
 }
 
 }  // namespace rlbm

@@ -205,12 +205,7 @@ __device__ __forceinline__ void pull_moments64(const typename S::T* __restrict__
   RLBM_PULL_DIR(4) RLBM_PULL_DIR(5) RLBM_PULL_DIR(6) RLBM_PULL_DIR(7)
   RLBM_PULL_DIR(8) RLBM_PULL_DIR(9) RLBM_PULL_DIR(10) RLBM_PULL_DIR(11)
 #undef RLBM_PULL_DIR
-  const Harm ha = harmonics(A, false), hb = harmonics(B, true);
-  N[0] = ha.h0; N[1] = ha.c1; N[2] = ha.s1;
-  T[0] = hb.h0; T[1] = hb.c1; T[2] = hb.s1;
-  T[3] = 0.5 * (hb.h0 + hb.c2);
-  T[4] = 0.5 * hb.s2;
-  T[5] = 0.5 * (hb.h0 - hb.c2);
+  moments_of(harmonics(A, false), harmonics(B, true), N, T);
 }
 
 // FP64 equilibrium at (theta, g, u) written through a functor out(q, value):
@@ -286,9 +281,9 @@ __device__ __forceinline__ int halo_targets(const DomDev& D, int x, int y, int h
 template <int EDF, class S>
 __device__ void write_halo64(const DomDev& D, int x, int y, typename S::T* __restrict__ fout, const double* sm,
                              int tid, bool have_state, double n, double ux, double uy, double gamma,
-                             unsigned& st, bool vw_written = false) {
+                             unsigned& st, bool vw_written = false, bool images = true) {
   int hx[8], hy[8], wall[8];
-  const int cnt = halo_targets(D, x, y, hx, hy, wall);
+  const int cnt = halo_targets(D, x, y, hx, hy, wall, images);
   for (int i = 0; i < cnt; ++i) {
     const long long h = cell_rel(D, hx[i], hy[i]);
     if (wall[i] >= 0 && D.bc[wall[i]] == BC_VWALL) {
@@ -320,47 +315,42 @@ __device__ __forceinline__ bool touches_vwall(const DomDev& D, int x, int y) {
 }
 
 // Velocity-wall ghosts of a cell (Sec. 3.4): f^eq(n_wall, 0, theta_wall) +
-// (f* - f^eq), f* the cell's post-collision populations (smem column) and f^eq
-// the equilibrium it relaxes towards -- its state (n, eps, theta, z) at the
-// force-shifted velocity u + a tau. At the initial state f* is the initial
-// equilibrium. Kept out of line: only edge cells pay for it.
-template <int EDF, class S>
-__device__ __noinline__ void write_vwall_ghosts(const DomDev& D, int x, int y, typename S::T* __restrict__ fout,
-                                                const double* sm, int tid, const CellState* cs, unsigned* st) {
-  int hx[8], hy[8], wall[8];
-  const int cnt = halo_targets(D, x, y, hx, hy, wall);
-  int tw_side = -1;
+// (f* - f^eq), f* the cell's post-collision populations and f^eq the equilibrium it
+// relaxes towards -- its state (n, eps, theta, z) at the force-shifted velocity
+// u + a tau. At the initial state f* is the initial equilibrium. The step holds f* and
+// f^eq shell by shell and writes the ghosts from them; the wall's own equilibrium, at
+// rest, has only its isotropic moments Z_n0 and is the same in every direction.
+struct VwallGhosts {
+  int cnt;             // ghost cells to write (0: none)
+  long long at[8];     // their element offsets
+  double y[6];         // Z_n0 of the wall state
+};
+
+template <int EDF>
+__device__ __noinline__ void vwall_setup(const DomDev& D, int x, int y, bool images, VwallGhosts* G, unsigned* st) {
+  int hx[8], hy[8], wall[8], side = -1;
+  const int cnt = halo_targets(D, x, y, hx, hy, wall, images);
+  G->cnt = 0;
   for (int i = 0; i < cnt; ++i)
-    if (wall[i] >= 0 && D.bc[wall[i]] == BC_VWALL) tw_side = wall[i];
-  if (tw_side < 0) return;
-  const double tw = D.t_wall[tw_side];  // shared by every velocity wall of the domain
-  const int oi = D.order - 2;
-  const double tau = D.eta_s > 0.0 ? 4.0 * D.eta_s / cs->theta + 0.2546 : D.tau;
-  double ux = cs->ux, uy = cs->uy, gam = cs->gamma;
-  if (D.accel_x != 0.0 || D.accel_y != 0.0) {
-    ux += D.accel_x * tau;
-    uy += D.accel_y * tau;
-    gam = 1.0 / sqrt(1.0 - ux * ux - uy * uy);
-  }
-  double z, g[6], yw[21], yc[21];
-  *st |= solve_z_from_n_theta<EDF, false>(D.n_wall, tw, z, g);
-  eq_moments<EDF>(g, tw, 0.0, 1.0, (2.0 * PI) * (tw * tw * g[1]), (4.0 * PI) * (tw * tw * tw) * g[2], yw, oi);
-  eq_moments<EDF>(cs->g, cs->theta, fma(ux, ux, uy * uy), gam, cs->n, cs->eps, yc, oi);
-  const DirPow Cw = dir_powers(0.0, 0.0), Cc = dir_powers(ux, uy);
-#pragma unroll 1
-  for (int s = 0; s < 6; ++s) {
-    double few[12], fe[12];
-    feq_shell<EDF>(s, yw, Cw, few, oi);
-    feq_shell<EDF>(s, yc, Cc, fe, oi);
-    for (int i = 0; i < cnt; ++i) {
-      if (wall[i] < 0 || D.bc[wall[i]] != BC_VWALL) continue;
-      const long long h = cell_rel(D, hx[i], hy[i]);
-      for (int d = 0; d < 12; ++d) {
-        const int q = 6 * d + s;
-        fout[plane_off(q) + h] = S::enc(few[d] + (sm[q * kThreads + tid] - fe[d]), D, s);
-      }
+    if (wall[i] >= 0 && D.bc[wall[i]] == BC_VWALL) {
+      side = wall[i];
+      G->at[G->cnt++] = cell_rel(D, hx[i], hy[i]);
     }
-  }
+  if (side < 0) return;
+  const double tw = D.t_wall[side];  // shared by every velocity wall of the domain
+  double z, g[6], yw[21];
+  *st |= solve_z_from_n_theta<EDF, false>(D.n_wall, tw, z, g);
+  eq_moments<EDF>(g, tw, 0.0, 1.0, (2.0 * PI) * (tw * tw * g[1]), (4.0 * PI) * (tw * tw * tw) * g[2], yw, D.order - 2);
+  for (int n = 0; n < 6; ++n) G->y[n] = yw[n * (n + 1) / 2];
+}
+
+// R_0 of shell s of the wall's equilibrium
+template <int EDF>
+__device__ __forceinline__ double vwall_shell(const VwallGhosts& G, int s, int oi) {
+  double a = c_Q[oi][EDF][s * 6] * G.y[0];
+#pragma unroll
+  for (int n = 1; n < 6; ++n) a = fma(c_Q[oi][EDF][s * 6 + n], G.y[n], a);
+  return a;
 }
 
 // The cell (x, y) of domain `dom` a thread of an initialiser or read-out
@@ -418,11 +408,23 @@ __global__ void __launch_bounds__(kThreads) k_init(InitArgs a) {
   }
   bool vw = false;
   if (ok && touches_vwall(D, x, y)) {
-    CellState cs;
-    cs.n = n; cs.theta = theta; cs.ux = ux; cs.uy = uy; cs.z = z; cs.gamma = gamma;
-    for (int k = 0; k < 6; ++k) cs.g[k] = g[k];
-    cs.eps = 4.0 * PI * theta * theta * theta * g[2];  // Eq. (25)
-    write_vwall_ghosts<EDF, S>(D, x, y, f, sm, tid, &cs, &st);
+    // f* is the initial equilibrium; f^eq the one at u + a tau
+    VwallGhosts G;
+    vwall_setup<EDF>(D, x, y, true, &G, &st);
+    const double tau = D.eta_s > 0.0 ? 4.0 * D.eta_s / theta + 0.2546 : D.tau;
+    const double vx = ux + D.accel_x * tau, vy = uy + D.accel_y * tau, v2 = fma(vx, vx, vy * vy);
+    double yc[21];
+    eq_moments<EDF>(g, theta, v2, 1.0 / sqrt(1.0 - v2), n, 4.0 * PI * theta * theta * theta * g[2], yc, D.order - 2);
+    const DirPow C = dir_powers(vx, vy);
+#pragma unroll 1
+    for (int s = 0; s < 6; ++s) {
+      double fe[12];
+      feq_shell<EDF>(s, yc, C, fe, D.order - 2);
+      const double fw = vwall_shell<EDF>(G, s, D.order - 2);
+      for (int i = 0; i < G.cnt; ++i)
+        for (int d = 0; d < 12; ++d)
+          f[G.at[i] + plane_off(6 * d + s)] = S::enc(fw + (sm[(6 * d + s) * kThreads + tid] - fe[d]), D, s);
+    }
     vw = true;
   }
   write_halo64<EDF, S>(D, x, y, f, sm, tid, ok, n, ux, uy, gamma, st, vw);
@@ -455,12 +457,7 @@ __global__ void __launch_bounds__(kThreads) k_fields(FieldsArgs a) {
       A[d] = a_;
       B[d] = b_;
     }
-    const Harm ha = harmonics(A, false), hb = harmonics(B, true);
-    N[0] = ha.h0; N[1] = ha.c1; N[2] = ha.s1;
-    T[0] = hb.h0; T[1] = hb.c1; T[2] = hb.s1;
-    T[3] = 0.5 * (hb.h0 + hb.c2);
-    T[4] = 0.5 * hb.s2;
-    T[5] = 0.5 * (hb.h0 - hb.c2);
+    moments_of(harmonics(A, false), harmonics(B, true), N, T);
   }
   CellState S_;
   unsigned st = cell_state<EDF, true>(N, T, S_);
