@@ -1030,8 +1030,9 @@ timed_out:
 // Macroscopic fields (n, theta, ux, uy, z) of a mixed storage's populations in
 // the collision's own arithmetic -- the FP32 pull and deviation sums, the
 // double-float totals and Landau frame (Eqs. 20-25), the FP32 fugacity solve --
-// written as FP64 (the double-float values exactly). It runs on the FP32 pipe;
-// the FP64 read-out k_fields, at 1/64 of that rate, serves the diagnostics.
+// written as FP64 (the double-float values to nearest). It runs on the FP32 pipe, the
+// conversions included (df_to_f64; on the FP64 unit they were a third of its time);
+// the FP64 read-out k_fields, at 1/64 of that rate, serves the diagnostics. Bound: HBM.
 template <int EDF, class S>
 __global__ void __launch_bounds__(kThreads) k_fields_mixed(FieldsArgs a) {
   int dom, x, y;
@@ -1040,6 +1041,7 @@ __global__ void __launch_bounds__(kThreads) k_fields_mixed(FieldsArgs a) {
   if (x >= D.nx || y >= D.ny) return;
   const typename S::T* __restrict__ f = static_cast<const typename S::T*>(a.f) + D.off;
   const long long c = cell_rel(D, x, y);
+  if (a.tiles && threadIdx.x == 0 && threadIdx.y == 0) prefetch_tile_l2<S>(D, a.tiles[blockIdx.x], f);
   f2 AB[12];
   {
     const PullW w = pull_weights<EDF, S>(D);
@@ -1077,11 +1079,11 @@ __global__ void __launch_bounds__(kThreads) k_fields_mixed(FieldsArgs a) {
       else theta = 0.5f * g[1] / g[2] * ef / nf;
     }
     const df ux = df_first(F.u), uy = df_second(F.u);
-    on = (double)F.n.hi + (double)F.n.lo;
-    oux = (double)ux.hi + (double)ux.lo;
-    ouy = (double)uy.hi + (double)uy.lo;
-    oth = theta;
-    oz = z;
+    on = df_to_f64(F.n);
+    oux = df_to_f64(ux);
+    ouy = df_to_f64(uy);
+    oth = f32_to_f64(theta);
+    oz = f32_to_f64(z);
   }
   const long long i = (a.tiles ? D.foff : 0) + (long long)y * D.nx + x;
   if (a.n) a.n[i] = on;
@@ -1139,6 +1141,8 @@ __global__ void __launch_bounds__(kThreads) k_init_mixed(InitArgs a) {
   const long long c = cell_rel(D, x, y);
   f2* col = reinterpret_cast<f2*>(smi) + tid;
   using P = Pair<typename S::T>;
+  // only warps with a cell on the domain's edge have halo cells to write
+  const bool edge_warp = __any_sync(__activemask(), x == 0 || x == D.nx - 1 || y == 0 || y == D.ny - 1);
   if (ok) {
     EqF q;
     dz_moments<EDF>(D, g, theta, ux, uy, gam, -1.0f, -1.0f, q);
@@ -1159,7 +1163,7 @@ __global__ void __launch_bounds__(kThreads) k_init_mixed(InitArgs a) {
       *reinterpret_cast<P*>(f + c + k * kSegW) = S::enc2(col[k * kThreads], D, 2 * (k % 3));
     }
   }
-  write_halo_mixed<EDF, S>(D, x, y, f, col, ok, n, ux, uy, gam, st, true);
+  if (edge_warp) write_halo_mixed<EDF, S>(D, x, y, f, col, ok, n, ux, uy, gam, st, true);
   if (st) atomicOr(a.status, st);
 }
 
