@@ -33,9 +33,33 @@ static __constant__ double c_E[4][3][18] = {
     {RLBM_EO4_MJ_INIT, RLBM_EO4_FD_INIT, RLBM_EO4_BE_INIT},
     {RLBM_E_MJ_INIT, RLBM_E_FD_INIT, RLBM_E_BE_INIT}};
 constexpr int kOrder5 = 3;  // table index of the fifth order
+// FP32 tables, rounded at compile time (a conversion in the kernel would take the FP64
+// unit): the same defects, for the correction itself (see eq_moments), the series of g_2
+// and g_3 in t, and the reversion t(w)
+struct TablesF {
+  float e[4][3][18], logser[2][12], rev[RLBM_NREV];
+};
+constexpr TablesF make_tables_f() {
+  constexpr double e[4][3][18] = {{RLBM_EO2_MJ_INIT, RLBM_EO2_FD_INIT, RLBM_EO2_BE_INIT},
+                                  {RLBM_EO3_MJ_INIT, RLBM_EO3_FD_INIT, RLBM_EO3_BE_INIT},
+                                  {RLBM_EO4_MJ_INIT, RLBM_EO4_FD_INIT, RLBM_EO4_BE_INIT},
+                                  {RLBM_E_MJ_INIT, RLBM_E_FD_INIT, RLBM_E_BE_INIT}};
+  constexpr double ls[5 * RLBM_NLOGSER] = RLBM_LOGSER_INIT;
+  constexpr double rv[RLBM_NREV] = RLBM_REV_INIT;
+  TablesF t{};
+  for (int i = 0; i < 12; ++i) {
+    t.logser[0][i] = (float)ls[i];
+    t.logser[1][i] = (float)ls[RLBM_NLOGSER + i];
+  }
+  for (int i = 0; i < RLBM_NREV; ++i) t.rev[i] = (float)rv[i];
+  for (int o = 0; o < 4; ++o)
+    for (int d = 0; d < 3; ++d)
+      for (int i = 0; i < 18; ++i) t.e[o][d][i] = (float)e[o][d][i];
+  return t;
+}
+static __constant__ TablesF c_tf = make_tables_f();
 static __constant__ double c_pnk[63] = RLBM_PNK_INIT;
 static __constant__ double c_logser[5 * RLBM_NLOGSER] = RLBM_LOGSER_INIT;
-static __constant__ double c_rev[RLBM_NREV] = RLBM_REV_INIT;
 static __constant__ double c_invpow[6 * RLBM_NSERIES] = RLBM_INVPOW_INIT;
 static __constant__ double c_be_exp[6 * RLBM_NEXP] = RLBM_BE_EXP_INIT;
 static __constant__ double c_fd_exp[6 * RLBM_NEXP] = RLBM_FD_EXP_INIT;
@@ -53,24 +77,44 @@ __host__ __device__ constexpr double pnk(int i) {
   return t[i];
 }
 
+// ------------------------------------- FP32 <-> FP64 on the integer pipe
+// The conversion instructions run on the FP64 unit too. Where an FP32 value only starts
+// or scales an FP64 correction, the bits are moved by integer instructions instead.
+// double -> float, cut towards zero; below the normal range 0, above it (and for
+// infinity and NaN) infinity
+__device__ __forceinline__ float cut_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), m = hi & 0x7fffffffu;
+  unsigned t = ((m - 0x38000000u) << 3) | (lo >> 29);
+  if (m < 0x38100000u) t = 0u;
+  if (m >= 0x47f00000u) t = 0x7f800000u;
+  return __uint_as_float(t | (hi & 0x80000000u));
+}
+// float -> double, exact for normal values and zeros; denormals go to 0. (Infinity and
+// NaN give a finite value: the caller's own test sends those states elsewhere.)
+__device__ __forceinline__ double widen_f64(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  return m < 0x00800000u ? __hiloint2double((int)(b & 0x80000000u), 0)
+                         : __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
 // ------------------------------------------------ FP64 divide and square root
 // GB300 issues one FP64 warp instruction per SM sub-partition every 64 clocks, so a
 // reciprocal or a root costs what its FP64 instructions cost. Both start from the
-// FP32 unit's value (about 24 bits) and take one step of a third-order (Halley)
+// FP32 unit's value (about 23 bits) and take one step of a third-order (Halley)
 // iteration in FP64: with e = 1 - x r, 1/x = r (1 + e + e^2 + ...), and with
 // e = 1 - x r^2, 1/sqrt(x) = r (1 + e/2 + 3 e^2/8 + ...); the terms left out are
-// below 2^-66. Outside the FP32 range they fall back to the compiler's own.
+// below 2^-64. Outside the FP32 range they fall back to the compiler's own.
 __device__ __forceinline__ double rcp64(double x) {
-  const float xf = (float)x;
+  const float xf = cut_f32(x);
   if (!(fabsf(xf) > 1e-30f && fabsf(xf) < 1e30f)) return 1.0 / x;
-  const double r = (double)(1.0f / xf);
+  const double r = widen_f64(1.0f / xf);
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
 __device__ __forceinline__ double rsqrt64(double x) {
-  const float xf = (float)x;
+  const float xf = cut_f32(x);
   if (!(xf > 1e-30f && xf < 1e30f)) return 1.0 / sqrt(x);
-  const double r = (double)rsqrtf(xf);
+  const double r = widen_f64(rsqrtf(xf));
   const double e = fma(-(x * r), r, 1.0);
   return fma(r * e, fma(0.375, e, 0.5), r);
 }
@@ -309,9 +353,9 @@ __device__ __forceinline__ void g23_t_f(float t, float& g2, float& g3) {
   const float u = EDF == EDF_BE ? t : -t, u2 = u * u;
   float a = 0.0f, b = 0.0f;
 #pragma unroll
-  for (int n = 10; n >= 2; n -= 2) a = fmaf(a, u2, (float)c_logser[n]);
+  for (int n = 10; n >= 2; n -= 2) a = fmaf(a, u2, c_tf.logser[0][n]);
 #pragma unroll
-  for (int n = 11; n >= 0; --n) b = fmaf(b, u, (float)c_logser[RLBM_NLOGSER + n]);
+  for (int n = 11; n >= 0; --n) b = fmaf(b, u, c_tf.logser[1][n]);
   g2 = t * fmaf(a, u2, fmaf(u, -0.25f, 1.0f));
   g3 = t * b;
 }
@@ -361,7 +405,7 @@ __device__ __forceinline__ double z_of_t(double t) { return EDF == EDF_BE ? -exp
 __device__ __forceinline__ void g_shift(double dmu, float g0, double g[6]) {
 #pragma unroll
   for (int i = 5; i >= 1; --i) g[i] = fma(dmu, g[i - 1], g[i]);
-  g[0] = fma(dmu, (double)g0, g[0]);
+  g[0] = fma(dmu, widen_f64(g0), g[0]);
 }
 
 // Fugacity from (eps, n), FD/BE: g_3^2/g_2^3 = target (Eq. 25). In t the ratio is
@@ -373,12 +417,12 @@ __device__ __forceinline__ void g_shift(double dmu, float g0, double g[6]) {
 // solver. kZ: z is wanted (the step only needs the g_nu).
 template <int EDF, bool kZ>
 __device__ __forceinline__ int solve_z_from_R(double target, double& z, double g[6]) {
-  const float wf = 1.0f / (float)target;
+  const float wf = 1.0f / cut_f32(target);
   if (wf > 1e-20f && wf < 1.25f) {
     const float sw = EDF == EDF_BE ? wf : -wf;
     float p = 0.0f;
 #pragma unroll
-    for (int n = RLBM_NREV - 1; n >= 0; --n) p = fmaf(p, sw, (float)c_rev[n]);
+    for (int n = RLBM_NREV - 1; n >= 0; --n) p = fmaf(p, sw, c_tf.rev[n]);
     float tf = wf * p;
     if (wf > 0.5f) {  // the reversion's own series is short there: two FP32 steps
 #pragma unroll
@@ -390,21 +434,21 @@ __device__ __forceinline__ int solve_z_from_R(double target, double& z, double g
     }
     if (tf > 0.0f && tf <= kTMax) {
       const int nt = logser_terms(tf);
-      double t = (double)tf, g2, g3;
+      double t = widen_f64(tf), g2, g3;
       g23_t<EDF>(t, nt, g2, g3);
       float g0 = g0_t_f<EDF>(tf);
       {
         const double a = target * (g2 * g2 * g2);
-        const float x = (float)fma(g3, g3, -a) / (float)a, r2 = (float)g2, r3 = (float)g3;
+        const float x = cut_f32(fma(g3, g3, -a)) / cut_f32(a), r2 = cut_f32(g2), r3 = cut_f32(g3);
         const float dmu = -x * fmaf(-0.5f, x, 1.0f) / (2.0f * r2 / r3 - 3.0f * tf / r2);
-        t += (double)(dmu * g0);
+        t += widen_f64(dmu * g0);
       }
       g_all_t<EDF>(t, nt, g);
       const double a = target * (g[1] * g[1] * g[1]);
-      const float r2 = (float)g[1], r3 = (float)g[2];
-      const float dmu = -((float)fma(g[2], g[2], -a) / (float)a) / (2.0f * r2 / r3 - 3.0f * tf / r2);
+      const float r2 = cut_f32(g[1]), r3 = cut_f32(g[2]);
+      const float dmu = -(cut_f32(fma(g[2], g[2], -a)) / cut_f32(a)) / (2.0f * r2 / r3 - 3.0f * tf / r2);
       if (fabsf(dmu) < 1e-9f) {
-        g_shift((double)dmu, g0, g);
+        g_shift(widen_f64(dmu), g0, g);
         if (kZ) z = z_of_t<EDF>(g[0]);
         return 0;
       }
@@ -424,7 +468,7 @@ __device__ __forceinline__ int solve_z_from_n_theta(double n, double theta, doub
     for (int i = 0; i < 6; ++i) g[i] = G;
     return 0;
   } else {
-    const float Gf = (float)G;
+    const float Gf = cut_f32(G);
     if (Gf > 1e-20f && Gf < 1.25f) {
       float tf = Gf * fmaf(Gf, fmaf(7.0f / 72.0f, Gf, EDF == EDF_BE ? 0.25f : -0.25f), 1.0f);
       if (EDF == EDF_BE) tf = fminf(tf, kTMax);
@@ -436,14 +480,14 @@ __device__ __forceinline__ int solve_z_from_n_theta(double n, double theta, doub
       }
       if (tf > 0.0f && tf <= kTMax) {
         const int nt = logser_terms(tf);
-        double t = (double)tf, g2, g3;
+        double t = widen_f64(tf), g2, g3;
         g23_t<EDF>(t, nt, g2, g3);
         const float g0 = g0_t_f<EDF>(tf);
-        t += (double)((float)(G - g2) * g0 / tf);
+        t += widen_f64(cut_f32(G - g2) * g0 / tf);
         g_all_t<EDF>(t, nt, g);
-        const float dmu = (float)(G - g[1]) / tf;
+        const float dmu = cut_f32(G - g[1]) / tf;
         if (fabsf(dmu) < 1e-9f) {
-          g_shift((double)dmu, g0, g);
+          g_shift(widen_f64(dmu), g0, g);
           if (kZ) z = z_of_t<EDF>(g[0]);
           return 0;
         }
@@ -503,8 +547,8 @@ static __device__ __noinline__ Frame landau_general(double E, double mx, double 
 // FP64 steps). States near the light cone or out of the
 // FP32 range, and any whose corrections do not shrink, take landau_general.
 __device__ __forceinline__ int landau(const double T[6], Frame& F) {
-  const float E = (float)T[0], mx = (float)T[1], my = (float)T[2], pxx = (float)T[3], pxy = (float)T[4],
-              pyy = (float)T[5];
+  const float E = cut_f32(T[0]), mx = cut_f32(T[1]), my = cut_f32(T[2]), pxx = cut_f32(T[3]), pxy = cut_f32(T[4]),
+              pyy = cut_f32(T[5]);
   const float disc = fmaf(9.0f * E, E, -8.0f * fmaf(mx, mx, my * my));
   if (E > 1e-15f && E < 1e15f && disc > 0.1f * E * E) {
     const float rx = 4.0f / fmaf(3.0f, E, sqrtf(disc));
@@ -524,15 +568,15 @@ __device__ __forceinline__ int landau(const double T[6], Frame& F) {
       fv = fmaf(fmaf(j10, fx, -j00 * fy), rdet, fv);
     }
     if (fmaf(fu, fu, fv * fv) < 0.95f) {
-      double ux = (double)fu, uy = (double)fv;
+      double ux = widen_f64(fu), uy = widen_f64(fv);
       float d = 0.0f;
       for (int it = 0; it < 6; ++it) {
         const double a = fma(-T[1], ux, fma(-T[2], uy, T[0]));
-        const float fx = (float)fma(-a, ux, fma(-T[3], ux, fma(-T[4], uy, T[1])));
-        const float fy = (float)fma(-a, uy, fma(-T[4], ux, fma(-T[5], uy, T[2])));
+        const float fx = cut_f32(fma(-a, ux, fma(-T[3], ux, fma(-T[4], uy, T[1]))));
+        const float fy = cut_f32(fma(-a, uy, fma(-T[4], ux, fma(-T[5], uy, T[2]))));
         const float dx = fmaf(j01, fy, -j11 * fx) * rdet, dy = fmaf(j10, fx, -j00 * fy) * rdet;
-        ux += (double)dx;
-        uy += (double)dy;
+        ux += widen_f64(dx);
+        uy += widen_f64(dy);
         d = fmaxf(fabsf(dx), fabsf(dy));
         if (d < 2e-11f) break;  // the next one would be below 1e-16
       }
@@ -642,17 +686,44 @@ __device__ __forceinline__ void eq_moments(const double g[6], double theta, doub
   // N^0, T^00 and T^0x, T^0y of f^eq equal Z_10, Z_20, Z_21 by the tiny constant
   // defects e1, e2, e3; correcting those three moments removes the resulting
   // bias (a constant error times Z would drift the conserved totals every step).
-  double d10 = 0.0, d20 = 0.0, d21 = 0.0;
+  // The corrections are below 2^-50 of the moments, so FP32 gives them to 2^-70.
+  float Af[6], big = 0.0f;
+  const float u2f = cut_f32(u2);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    d10 = fma(c_E[oi][EDF][k], y[k * (k + 1) / 2], d10);
-    d20 = fma(c_E[oi][EDF][6 + k], y[k * (k + 1) / 2], d20);
+    Af[k] = cut_f32(A[k]);
+    big = fmaxf(big, fabsf(Af[k]));
   }
+  if (big < 1e30f && big > 1e-15f) {
+    float d10 = 0.0f, d20 = 0.0f, d21 = 0.0f;
 #pragma unroll
-  for (int k = 1; k < 6; ++k) d21 = fma(c_E[oi][EDF][12 + k], y[k * (k + 1) / 2 + 1], d21);
-  y[1] -= d10;
-  y[3] -= d20;
-  y[4] -= d21;
+    for (int n_ = 0; n_ < 6; ++n_) {
+#pragma unroll
+      for (int k = 0; k <= (n_ ? 1 : 0); ++k) {
+        const int i = 3 * (n_ * (n_ + 1) / 2 + k);
+        const float yf = Af[n_] * fmaf(u2f, fmaf(u2f, (float)pnk(i + 2), (float)pnk(i + 1)), (float)pnk(i));
+        if (k == 0) {
+          d10 = fmaf(c_tf.e[oi][EDF][n_], yf, d10);
+          d20 = fmaf(c_tf.e[oi][EDF][6 + n_], yf, d20);
+        } else {
+          d21 = fmaf(c_tf.e[oi][EDF][12 + n_], yf, d21);
+        }
+      }
+    }
+    y[1] -= widen_f64(d10);
+    y[3] -= widen_f64(d20);
+    y[4] -= widen_f64(d21);
+  } else {  // moments outside the FP32 range
+    double d10 = 0.0, d20 = 0.0, d21 = 0.0;
+    for (int k = 0; k < 6; ++k) {
+      d10 = fma(c_E[oi][EDF][k], y[k * (k + 1) / 2], d10);
+      d20 = fma(c_E[oi][EDF][6 + k], y[k * (k + 1) / 2], d20);
+      if (k) d21 = fma(c_E[oi][EDF][12 + k], y[k * (k + 1) / 2 + 1], d21);
+    }
+    y[1] -= d10;
+    y[3] -= d20;
+    y[4] -= d21;
+  }
 }
 
 // C_k(d) = Re[(u_x + i u_y)^k e^{-i k phi_d}] of the directions d = 0..5 (d + 6

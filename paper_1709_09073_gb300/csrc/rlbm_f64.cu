@@ -31,19 +31,16 @@ __device__ __forceinline__ void collision_frame(const DomDev& D, double theta, d
 //
 // Bound: the FP64 pipe. One FP64 warp instruction holds its SM sub-partition's unit
 // for 64 clocks, whatever its operation and however many lanes are active, so the
-// count of FP64 instructions per cell is the time. About 1,040 (MJ): pull 192, moments
-// 200, Landau 40 (FP32 start), state and equilibrium moments 90, directional powers
+// count of FP64 instructions per cell is the time. About 1,000 (MJ): pull 192, moments
+// 200, Landau 35 (FP32 start), state and equilibrium moments 65, directional powers
 // and rates 45, six shells of 80 (21 projection, 35 synthesis, 24 relaxation). With
 // FP64 Newton throughout and harmonic powers applied before the projection it was
-// 1,382. 512^2 local-tau disc, 8 steps with initialisation and read-out: 6.00 -> 4.54
-// ms; FD Riemann 2048 x 4, 50 steps: 5.89 -> 3.12 ms; BE 1024^2, 4 steps: 21.6 -> 11.5 ms.
+// 1,382; conversions (the FP64 unit's too) run on the integer pipe. A 512^2 domain a
+// step: MJ 720 -> 513 us, BE 1,000 -> 568 us; the local-tau disc 730 -> 525 us.
 // kVw: the launch has velocity walls (StepArgs::halo 3); without them their code and its
-// registers are left out (512^2: 569 -> 540 us).
-#ifndef RLBM_F64_BLOCKS
-#define RLBM_F64_BLOCKS 2
-#endif
+// registers are left out (512^2: 569 -> 530 us).
 template <int EDF, bool kVw>
-__global__ void __launch_bounds__(kThreads, RLBM_F64_BLOCKS) k_step_f64(StepArgs a) {
+__global__ void __launch_bounds__(kThreads, 2) k_step_f64(StepArgs a) {
   extern __shared__ double sm[];
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
@@ -118,8 +115,9 @@ __global__ void __launch_bounds__(kThreads, RLBM_F64_BLOCKS) k_step_f64(StepArgs
 // pulls, sums, relaxes and stores the directions 2W, 2W + 1 and their opposites; the
 // Landau solve runs in one warp (a different one from block to block); then that
 // warp forms the equilibrium moments while the next forms the directional powers;
-// each warp projects two shells. About 510 instructions in the longest chain instead
-// of 1,040. 64^2, one domain alone: 48 -> 26 us a step.
+// each warp projects two shells. About 490 instructions in the longest chain instead
+// of 1,000. One domain alone, a step: 64^2 44 -> 20.8 us, FD Riemann 2048 x 4 55 -> 35 us,
+// 8 x 255 channel 57 -> 37 us.
 struct SplitSm {
   double eo[6][4][32];     // e, o of A and B (harmonics_eo) per direction pair
   double cell[6][32];      // u_x, u_y, gamma, n, eps, theta
@@ -411,13 +409,11 @@ cudaError_t prepare_f64() {
 // Most tiles of a launch that takes the split step (at one block per tile): 4 blocks of
 // it per tile, two on each of 152 SMs. Measured, plain / split, us a step (MJ): 32^2 47.4 /
 // 21.5, 64^2 47.4 / 21.8, 96^2 (72 tiles) 47.4 / 27.5, 112^2 (98) 47.4 / 50.7, 256^2 164 / 171.
-#ifndef RLBM_SPLIT_TILES
-#define RLBM_SPLIT_TILES 76
-#endif
+constexpr int kSplitTiles = 76;
 
 template <int EDF, bool kVw>
 static void launch_step_t(const StepArgs& a, int grid, cudaStream_t s) {
-  if (grid == a.ntiles && a.ntiles <= RLBM_SPLIT_TILES)
+  if (grid == a.ntiles && a.ntiles <= kSplitTiles)
     k_step_f64_split<EDF, kVw><<<grid * kTileH, dim3(32, kSplitWarps), 0, s>>>(a);
   else
     k_step_f64<EDF, kVw><<<grid, dim3(kTileW, kTileH), kSmem64, s>>>(a);
