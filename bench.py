@@ -322,11 +322,11 @@ def run_native(args):
 
 
 # FP64 operations per cell update of the plain kernel (k_step_f64<MJ>), FMA = 2:
-# 872 DFMA + 308 DADD + 202 DMUL per cell, the executed-instruction counts ncu
+# 662 DFMA + 201 DADD + 146 DMUL per cell, the executed-instruction counts ncu
 # reports for one 1024^2 launch divided by its cells; used for the FP64 ALU
 # roofline of the plain form.
-FP64_FLOPS_PER_CELL = 2 * 872 + 308 + 202
-FP64_INSTR_PER_CELL = 872 + 308 + 202
+FP64_FLOPS_PER_CELL = 2 * 662 + 201 + 146
+FP64_INSTR_PER_CELL = 662 + 201 + 146
 
 
 def _oracle_rate(O, wl, budget_s):

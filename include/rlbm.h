@@ -133,8 +133,8 @@ size_t rlbm_workspace_bytes(const rlbm_config *config);
 
 /* The tile work list a handle of this configuration would walk (host only, no
  * device work; the paper has no counterpart): packed = 0 the plain list of
- * 32 x 4 tiles (TMA-staged and FP64 steps, initialisers, read-outs), packed = 1
- * the list of the mixed L1 step, where each domain's ragged last x block of
+ * 32 x 4 tiles (TMA-staged step, initialisers, read-outs), packed = 1
+ * the list of the FP64 and the mixed L1 steps, where each domain's ragged last x block of
  * w <= 16 cells is one tile per 4 * (32 / w) rows, a warp covering 32 / w rows
  * of w cells. Writes up to max_tiles quadruples (domain, x0, y0, w) to `out`
  * (host, int[4 * max_tiles]; may be null) and returns the number of tiles, or
@@ -194,8 +194,8 @@ int rlbm_moments_all(rlbm_handle h, int streamed, double *n, double *theta, doub
 int rlbm_diagnostics(rlbm_handle h, int domain, int streamed, double *out, int on_device);
 
 /* Raw state of domain `domain` for checkpoint/resume: the stored populations
- * including the one-cell halo ring (periodic images, which the mixed L1 step
- * does not store, are filled from the interior first), as FP64 [72][ny+2][nx+2] (index
+ * including the one-cell halo ring (periodic images, which the FP64 and the
+ * mixed L1 steps do not store, are filled from the interior first), as FP64 [72][ny+2][nx+2] (index
  * (q*(ny+2) + y+1)*(nx+2) + x+1 for x in -1..nx, y in -1..ny), converted from
  * the storage format. rlbm_set_populations writes them back (rounded to the
  * storage format); a resumed run then continues bit-for-bit. */
@@ -248,7 +248,7 @@ int rlbm_tune(rlbm_handle h, int repeats);
 
 /* Launch the step kernel with `grid` blocks in later rlbm_step calls: a
  * persistent grid, each block walking the tile list with stride `grid`, or
- * one block per tile for grid = 0 (the default). The mixed L1 step walks a
+ * one block per tile for grid = 0 (the default). The FP64 and the mixed L1 steps walk a
  * list in which each domain's ragged last block of w <= 16 cells is packed,
  * 32 / w rows per warp; the other kernels walk 32 x 4 tiles. rlbm_tune sets it
  * as well. Returns the grid now in use (grid >= 0) or RLBM_E_ARG. */
