@@ -871,12 +871,13 @@ __device__ __forceinline__ void step_tile_mixed(const StepArgs& a, int t, float*
 // kHalo = StepArgs::halo (see collide_mixed): 0 no halo writer, 0 and 1 no copy
 // of the relaxed values into the column.
 //
-// Bound: HBM for the FP32 storages (2048^2 periodic, FP32 deviations: 378 us, 6.39
-// TB/s of algorithmic traffic, 0.94 of the copy rate), instructions and load latency
-// for the 16-bit ones (332 us, 0.54 of it). Planes in pairs: one load or store moves
+// Bound: HBM for the FP32 storages (2048^2 periodic, FP32 deviations: 376 us, 6.42
+// TB/s of algorithmic traffic, 0.94 of the copy rate), instructions and the FP32 pipe
+// for the 16-bit ones (328 us, 0.54 of it). Planes in pairs: one load or store moves
 // the shells s, s + 1 of a direction, and the pull, the sums and the synthesis work on
 // them as f32x2. With one plane per segment and scalar arithmetic the same step
-// issued about twice the instructions: 461 us (FP32 deviations), 500 us (BF16).
+// issued 1.6 times the instructions (2,774 per 32 cells, now 1,702): 461 us (FP32
+// deviations), 500 us (BF16).
 template <int EDF, class S, int kHalo>
 __global__ void __launch_bounds__(kThreads, (mixed_min_blocks<S, kHalo>())) k_step_mixed(StepArgs a) {
   extern __shared__ float smf[];
