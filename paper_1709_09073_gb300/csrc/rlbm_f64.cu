@@ -165,7 +165,7 @@ __device__ __forceinline__ void split_pull(const double* __restrict__ fin, long 
   }
 }
 
-// Relaxation of a warp's directions: v becomes f*; `fe`, the equilibria, for velocity walls.
+// Relaxation of a warp's directions: v becomes f*; ghost(d, s, f*, f^eq) writes velocity-wall ghosts.
 template <int EDF, int W, class Ghost>
 __device__ __forceinline__ void split_relax(double K, double v[4][6], const SplitSm& sm, int lane, Ghost ghost) {
   DirPow C;  // the entries of directions 2W, 2W + 1

@@ -99,7 +99,6 @@ constexpr float kPIf = 3.14159265358979f;
 constexpr float kH = 0.866025403784438647f;
 constexpr float kHl = (float)(0.866025403784438647 - (double)kH);
 __device__ __forceinline__ float mul_h(float x) { return fmaf(kH, x, kHl * x); }
-__device__ __forceinline__ float fma_h(float x, float y) { return fmaf(kH, x, fmaf(kHl, x, y)); }
 constexpr float kRZCf = (float)RLBM_R_ZC;
 constexpr float kZCf = 0.9999999f;
 
