@@ -364,23 +364,23 @@ __device__ __forceinline__ void g23_t_f(float t, float& g2, float& g3) {
 template <int EDF>
 __device__ __forceinline__ float g0_t_f(float t) { return EDF == EDF_BE ? expm1f(t) : -expm1f(-t); }
 
-// g_2 (even terms beyond the second vanish, Li_2 - u + u^2/4 being odd) and g_3
+// h_2 and h_3 of g_nu = t h_nu (even terms of h_2 beyond the second vanish, Li_2 - u +
+// u^2/4 being odd)
 template <int EDF>
-__device__ __forceinline__ void g23_t(double t, int nt, double& g2, double& g3) {
+__device__ __forceinline__ void h23_t(double t, int nt, double& h2, double& h3) {
   const double u = EDF == EDF_BE ? t : -t, u2 = u * u;
   double a = 0.0, b = 0.0;
   for (int n = nt; n >= 2; n -= 2) {
     a = fma(a, u2, c_logser[n]);
     b = fma(fma(b, u, c_logser[RLBM_NLOGSER + n + 1]), u, c_logser[RLBM_NLOGSER + n]);
   }
-  b = fma(fma(b, u, c_logser[RLBM_NLOGSER + 1]), u, c_logser[RLBM_NLOGSER]);
-  g2 = t * fma(a, u2, fma(u, -0.25, 1.0));
-  g3 = t * b;
+  h2 = fma(a, u2, fma(u, -0.25, 1.0));
+  h3 = fma(fma(b, u, c_logser[RLBM_NLOGSER + 1]), u, c_logser[RLBM_NLOGSER]);
 }
 
-// all six (g_1 = t)
+// h[nu - 1] of all six (h_1 = 1)
 template <int EDF>
-__device__ __forceinline__ void g_all_t(double t, int nt, double g[6]) {
+__device__ __forceinline__ void h_all_t(double t, int nt, double h[6]) {
   const double u = EDF == EDF_BE ? t : -t, u2 = u * u;
   double a = 0.0, b[4] = {0.0, 0.0, 0.0, 0.0};
   for (int n = nt; n >= 2; n -= 2) {
@@ -389,32 +389,34 @@ __device__ __forceinline__ void g_all_t(double t, int nt, double g[6]) {
     for (int j = 0; j < 4; ++j)
       b[j] = fma(fma(b[j], u, c_logser[(j + 1) * RLBM_NLOGSER + n + 1]), u, c_logser[(j + 1) * RLBM_NLOGSER + n]);
   }
-  g[0] = t;
-  g[1] = t * fma(a, u2, fma(u, -0.25, 1.0));
+  h[0] = 1.0;
+  h[1] = fma(a, u2, fma(u, -0.25, 1.0));
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    g[2 + j] = t * fma(fma(b[j], u, c_logser[(j + 1) * RLBM_NLOGSER + 1]), u, c_logser[(j + 1) * RLBM_NLOGSER]);
+    h[2 + j] = fma(fma(b[j], u, c_logser[(j + 1) * RLBM_NLOGSER + 1]), u, c_logser[(j + 1) * RLBM_NLOGSER]);
 }
 
 // z of t
 template <int EDF>
 __device__ __forceinline__ double z_of_t(double t) { return EDF == EDF_BE ? -expm1(-t) : expm1(t); }
 
-// g_nu moved by a step dmu of ln z that is below 1e-9: dg_nu/dmu = g_(nu-1), the
-// second-order term is below 1e-18.
-__device__ __forceinline__ void g_shift(double dmu, float g0, double g[6]) {
+// g_nu a step dmu of ln z (below 1e-9) beyond t: dg_nu/dmu = g_(nu-1), the second-order
+// term is below 1e-18.
+__device__ __forceinline__ void g_shift(double t, double dmu, float g0, const double h[6], double g[6]) {
 #pragma unroll
-  for (int i = 5; i >= 1; --i) g[i] = fma(dmu, g[i - 1], g[i]);
-  g[0] = fma(dmu, widen_f64(g0), g[0]);
+  for (int i = 5; i >= 1; --i) g[i] = t * fma(dmu, h[i - 1], h[i]);
+  g[0] = fma(dmu, widen_f64(g0), t);
 }
 
 // Fugacity from (eps, n), FD/BE: g_3^2/g_2^3 = target (Eq. 25). In t the ratio is
 // w = 1/target = g_2^3/g_3^2 = t - (47/1728) t^3 - ..., so the reversion gives t to
 // FP32 accuracy; one FP64 Newton step (in mu = ln z, whose F' = 2 g_2/g_3 - 3 g_1/g_2
 // may be FP32) leaves about 1e-13, and the second one, taken from the residual at
-// that point and carried to the six g_nu to first order, about 1e-20. States outside
-// the series' range, and any whose second step is not small, take the general
-// solver. kZ: z is wanted (the step only needs the g_nu).
+// that point and carried to the six g_nu to first order, about 1e-20. Both residuals are
+// formed with t divided out, from h_2, h_3 and w/t, all of order one: the squares of the
+// g_nu leave the FP32 range below t = 1e-12, where a residual cut to zero would pass for
+// a converged one. States outside the series' range, and any whose second step is not
+// small, take the general solver. kZ: z is wanted (the step only needs the g_nu).
 template <int EDF, bool kZ>
 __device__ __forceinline__ int solve_z_from_R(double target, double& z, double g[6]) {
   const float wf = 1.0f / cut_f32(target);
@@ -434,21 +436,21 @@ __device__ __forceinline__ int solve_z_from_R(double target, double& z, double g
     }
     if (tf > 0.0f && tf <= kTMax) {
       const int nt = logser_terms(tf);
-      double t = widen_f64(tf), g2, g3;
-      g23_t<EDF>(t, nt, g2, g3);
-      float g0 = g0_t_f<EDF>(tf);
+      double t = widen_f64(tf), h2, h3, h[6];
+      h23_t<EDF>(t, nt, h2, h3);
+      const float g0 = g0_t_f<EDF>(tf);
       {
-        const double a = target * (g2 * g2 * g2);
-        const float x = cut_f32(fma(g3, g3, -a)) / cut_f32(a), r2 = cut_f32(g2), r3 = cut_f32(g3);
-        const float dmu = -x * fmaf(-0.5f, x, 1.0f) / (2.0f * r2 / r3 - 3.0f * tf / r2);
+        const double a = (target * t) * (h2 * h2 * h2);
+        const float x = cut_f32(fma(h3, h3, -a)) / cut_f32(a), r2 = cut_f32(h2), r3 = cut_f32(h3);
+        const float dmu = -x * fmaf(-0.5f, x, 1.0f) / (2.0f * r2 / r3 - 3.0f / r2);
         t += widen_f64(dmu * g0);
       }
-      g_all_t<EDF>(t, nt, g);
-      const double a = target * (g[1] * g[1] * g[1]);
-      const float r2 = cut_f32(g[1]), r3 = cut_f32(g[2]);
-      const float dmu = -(cut_f32(fma(g[2], g[2], -a)) / cut_f32(a)) / (2.0f * r2 / r3 - 3.0f * tf / r2);
+      h_all_t<EDF>(t, nt, h);
+      const double a = (target * t) * (h[1] * h[1] * h[1]);
+      const float r2 = cut_f32(h[1]), r3 = cut_f32(h[2]);
+      const float dmu = -(cut_f32(fma(h[2], h[2], -a)) / cut_f32(a)) / (2.0f * r2 / r3 - 3.0f / r2);
       if (fabsf(dmu) < 1e-9f) {
-        g_shift(widen_f64(dmu), g0, g);
+        g_shift(t, widen_f64(dmu), g0, h, g);
         if (kZ) z = z_of_t<EDF>(g[0]);
         return 0;
       }
@@ -480,14 +482,14 @@ __device__ __forceinline__ int solve_z_from_n_theta(double n, double theta, doub
       }
       if (tf > 0.0f && tf <= kTMax) {
         const int nt = logser_terms(tf);
-        double t = widen_f64(tf), g2, g3;
-        g23_t<EDF>(t, nt, g2, g3);
+        double t = widen_f64(tf), h2, h3, h[6];
+        h23_t<EDF>(t, nt, h2, h3);
         const float g0 = g0_t_f<EDF>(tf);
-        t += widen_f64(cut_f32(G - g2) * g0 / tf);
-        g_all_t<EDF>(t, nt, g);
-        const float dmu = cut_f32(G - g[1]) / tf;
+        t += widen_f64(cut_f32(fma(-t, h2, G)) * g0 / tf);
+        h_all_t<EDF>(t, nt, h);
+        const float dmu = cut_f32(fma(-t, h[1], G)) / tf;
         if (fabsf(dmu) < 1e-9f) {
-          g_shift(widen_f64(dmu), g0, g);
+          g_shift(t, widen_f64(dmu), g0, h, g);
           if (kZ) z = z_of_t<EDF>(g[0]);
           return 0;
         }

@@ -223,7 +223,7 @@ __device__ __forceinline__ bool newton_done(float d, float z) {
 }
 
 // The six g_nu of t = g_1 <= 0.5 (z = 0.65 FD, 0.39 BE): nine terms put the first one
-// left out below 1e-9 of the sum; no logarithm, no exponential (see g_all_t).
+// left out below 1e-9 of the sum; no logarithm, no exponential (see h_all_t).
 template <int EDF>
 __device__ __forceinline__ void g_all_tf(float t, float g[6]) {
   const float u = EDF == EDF_BE ? t : -t, u2 = u * u;
