@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_step_f64(StepArgs a) {
       // a clamped BE state relaxes to its own equilibrium energy 4 pi theta^3 g_3(z_c)
       const double eps_eq = (st & ST_CLAMPED) ? 4.0 * PI * S.theta * S.theta * S.theta * S.g[2] : S.eps;
       eq_moments<EDF>(S.g, S.theta, fma(ux, ux, uy * uy), gam, S.n, eps_eq, ym, oi);
-      const bool vw = kVw && touches_vwall(D, x, y);
+      const bool vw = kVw && touches_vwall(D, x, y), clamped = (st & ST_CLAMPED) != 0;
       VwallGhosts G;
       if (vw) vwall_setup<EDF>(D, x, y, a.images != 0, &G, &st);
 #pragma unroll 1
@@ -96,6 +96,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_step_f64(StepArgs a) {
           }
         }
       }
+      if (EDF == EDF_BE && vw && clamped)
+        vwall_clamped<true>(D, &G, S.theta, S.n, S.eps, ux, uy, gam, sm + tid, 0xfffu, fout);
     }
     // f* (or the unrelaxed populations of a non-physical cell), a plane pair per store
 #pragma unroll 4
@@ -124,7 +126,7 @@ struct SplitSm {
   double y[21][32];        // equilibrium moments
   double c[20][32];        // DirPow
   double R[6][6][32];      // projection by shell, k
-  unsigned st[32];
+  unsigned st[32], clamped[32];
 };
 constexpr int kSplitWarps = 3;
 
@@ -297,6 +299,7 @@ __device__ __forceinline__ void split_cell(const StepArgs& a, const DomDev& D, i
   if (ok && serial == W) {
     st |= cell_theta<EDF, false>(S);
     sm.cell[5][lane] = S.theta;
+    sm.clamped[lane] = st & ST_CLAMPED;
   }
   if (D.eta_s > 0.0) split_sync();  // every warp's rate needs theta (uniform per domain)
   if (ok) {
@@ -339,8 +342,8 @@ __device__ __forceinline__ void split_cell(const StepArgs& a, const DomDev& D, i
   }
   split_sync();
   const bool vw = kVw && in && ok && touches_vwall(D, x, y);
+  VwallGhosts G;
   if (kVw && __any_sync(0xffffffffu, vw)) {
-    VwallGhosts G;
     G.cnt = 0;
     if (vw) vwall_setup<EDF>(D, x, y, a.images != 0, &G, &st);
     if (ok)
@@ -354,6 +357,9 @@ __device__ __forceinline__ void split_cell(const StepArgs& a, const DomDev& D, i
   }
   if (in) {
     split_store<W>(fout, c, v);
+    if (EDF == EDF_BE && vw && sm.clamped[lane])
+      vwall_clamped<false>(D, &G, sm.cell[5][lane], sm.cell[3][lane], sm.cell[4][lane], ux, uy, gam, fout + c,
+                           0xc3u << (2 * W), fout);
     const bool edge = x == 0 || x == D.nx - 1 || y == 0 || y == D.ny - 1;
     if (edge && (a.images || a.halo)) {
       double n = 0.0, hx = 0.0, hy = 0.0, hg = 1.0;

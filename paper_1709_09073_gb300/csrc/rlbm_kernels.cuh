@@ -353,6 +353,33 @@ __device__ __forceinline__ double vwall_shell(const VwallGhosts& G, int s, int o
   return a;
 }
 
+// The same ghosts of a clamped BE cell, which relaxes to the energy of the equilibrium at
+// z_c instead of its own: its ghosts are measured against the equilibrium of its own n and
+// eps (as the oracle does), at the velocity (ux, uy, gamma) the collision used. f* of plane
+// q is at fs[q * kThreads] (kColumn) or fs[plane_off(q)]; the directions whose bits are set
+// in dirs.
+template <bool kColumn>
+__device__ __noinline__ void vwall_clamped(const DomDev& D, const VwallGhosts* G, double theta, double n, double eps,
+                                           double ux, double uy, double gamma, const double* fs, unsigned dirs,
+                                           double* fout) {
+  double y[21];
+  eq_moments<EDF_BE>(c_g_zc, theta, fma(ux, ux, uy * uy), gamma, n, eps, y, D.order - 2);
+  const DirPow C = dir_powers(ux, uy);
+#pragma unroll 1
+  for (int s = 0; s < 6; ++s) {
+    double fe[12];
+    feq_shell<EDF_BE>(s, y, C, fe, D.order - 2);
+    const double fw = vwall_shell<EDF_BE>(*G, s, D.order - 2);
+#pragma unroll
+    for (int d = 0; d < 12; ++d) {
+      if (!(dirs >> d & 1)) continue;
+      const int q = 6 * d + s;
+      const double g = fw + (fs[kColumn ? q * kThreads : plane_off(q)] - fe[d]);
+      for (int i = 0; i < G->cnt; ++i) fout[G->at[i] + plane_off(q)] = g;
+    }
+  }
+}
+
 // The cell (x, y) of domain `dom` a thread of an initialiser or read-out
 // launch covers: a block per tile of the work list, or a 2D grid over one domain.
 __device__ __forceinline__ void cell_of_launch(const Tile* tiles, int dom0, int& dom, int& x, int& y) {
