@@ -239,7 +239,7 @@ int rlbm_unpack_ghost_rows(rlbm_handle h, int domain, const void *lo, const void
 
 /* Autotune the launch of the step kernel on the current state (left unchanged):
  * time `repeats` launches of each candidate -- every kernel variant the handle
- * has (rlbm_select_kernel) with one block per 32 x 4 tile or a persistent grid
+ * has (rlbm_select_kernel) with one block per tile (grid = 0) or a persistent grid
  * of k x (SM count) blocks, k in {1, 2, 3, 4, 6, 8} -- and keep the fastest for
  * later rlbm_step calls (the captured step graphs are rebuilt). Every domain
  * must be initialised. Returns the chosen grid size (> 0) or an error; device
@@ -248,7 +248,9 @@ int rlbm_tune(rlbm_handle h, int repeats);
 
 /* Launch the step kernel with `grid` blocks in later rlbm_step calls: a
  * persistent grid, each block walking the tile list with stride `grid`, or
- * one block per tile for grid = 0 (the default). The FP64 and the mixed L1 steps walk a
+ * one block per tile for grid = 0 (the default; an FP64 launch of at most 76 tiles then
+ * takes the step of few tiles, three warps on each row of a tile, with the same results).
+ * The FP64 and the mixed L1 steps walk a
  * list in which each domain's ragged last block of w <= 16 cells is packed,
  * 32 / w rows per warp; the other kernels walk 32 x 4 tiles. rlbm_tune sets it
  * as well. Returns the grid now in use (grid >= 0) or RLBM_E_ARG. */

@@ -230,9 +230,8 @@ cudaError_t launch_step(rlbm_ctx* h, int from) {
   a.wait_ns = h->wait_ns;
   a.halo = h->halo;
   a.images = 0;
-  const int grid = h->grid > 0 ? h->grid : a.ntiles;
-  if (h->storage == RLBM_F64) return launch_step_f64(h->edf, a, grid, h->stream);
-  return launch_step_mixed(h->storage, h->edf, a, grid, h->stream);
+  if (h->storage == RLBM_F64) return launch_step_f64(h->edf, a, h->grid, h->stream);
+  return launch_step_mixed(h->storage, h->edf, a, h->grid > 0 ? h->grid : a.ntiles, h->stream);
 }
 
 // Capture `nsteps` (even) steps starting from copy `from` into an executable graph.
@@ -809,7 +808,8 @@ int rlbm_tune(rlbm_handle h, int repeats) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return RLBM_E_CUDA;
-  // grid 0: one block per tile of whichever list the variant walks
+  // grid 0: one block per tile of whichever list the variant walks (or the FP64 step of
+  // few tiles)
   const int ntiles = (int)h->L.stiles().size();
   std::vector<int> cand = {0};
   for (int k : {1, 2, 3, 4, 6, 8})

@@ -412,17 +412,17 @@ cudaError_t prepare_f64() {
   return prepare_t<EDF_BE>();
 }
 
-// Most tiles of a launch that takes the split step (at one block per tile): 4 blocks of
+// Most tiles of a launch that takes the split step (unless a grid is asked for): 4 blocks of
 // it per tile, two on each of 152 SMs. Measured, plain / split, us a step (MJ): 32^2 47.4 /
 // 21.5, 64^2 47.4 / 21.8, 96^2 (72 tiles) 47.4 / 27.5, 112^2 (98) 47.4 / 50.7, 256^2 164 / 171.
 constexpr int kSplitTiles = 76;
 
 template <int EDF, bool kVw>
 static void launch_step_t(const StepArgs& a, int grid, cudaStream_t s) {
-  if (grid == a.ntiles && a.ntiles <= kSplitTiles)
-    k_step_f64_split<EDF, kVw><<<grid * kTileH, dim3(32, kSplitWarps), 0, s>>>(a);
+  if (grid == 0 && a.ntiles <= kSplitTiles)
+    k_step_f64_split<EDF, kVw><<<a.ntiles * kTileH, dim3(32, kSplitWarps), 0, s>>>(a);
   else
-    k_step_f64<EDF, kVw><<<grid, dim3(kTileW, kTileH), kSmem64, s>>>(a);
+    k_step_f64<EDF, kVw><<<grid > 0 ? grid : a.ntiles, dim3(kTileW, kTileH), kSmem64, s>>>(a);
 }
 
 cudaError_t launch_step_f64(int edf, const StepArgs& a, int grid, cudaStream_t s) {

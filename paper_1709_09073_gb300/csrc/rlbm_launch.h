@@ -41,6 +41,8 @@ struct CopyArgs {
 
 // FP64 storage (plain method)
 cudaError_t prepare_f64();
+// grid > 0: a persistent grid of that many blocks; 0: one block per tile, or the step of
+// few tiles
 cudaError_t launch_step_f64(int edf, const StepArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_init_f64(int edf, const InitArgs& a, int nx, int ny, cudaStream_t s);
 cudaError_t launch_fields_f64(int edf, const FieldsArgs& a, int nx, int ny, cudaStream_t s);

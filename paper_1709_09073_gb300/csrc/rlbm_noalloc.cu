@@ -186,7 +186,7 @@ extern "C" int rlbm_step_noalloc(const rlbm_domain* domain, int edf, int nsteps,
     a.wait_ns = 0;
     a.halo = 3;  // any side
     a.images = 1;  // f_out holds the whole halo
-    e = launch_step_f64(edf, a, P.ntiles, s);
+    e = launch_step_f64(edf, a, 0, s);
     cur = 1 - cur;
   }
   if (e == cudaSuccess) {  // halo-padded copy -> checkpoint layout
