@@ -455,7 +455,7 @@ int rlbm_layout_tiles(const rlbm_config* c, int packed, int* out, int max_tiles)
   if (validate(c) || max_tiles < 0) return RLBM_E_ARG;
   Layout L;
   make_layout(c, L);
-  const std::vector<Tile>& t = packed ? L.ptiles : L.tiles;
+  const std::vector<Tile>& t = packed ? L.stiles() : L.tiles;
   if (out)
     for (size_t i = 0; i < t.size() && (long long)i < max_tiles; ++i) {
       out[4 * i + 0] = t[i].dom;

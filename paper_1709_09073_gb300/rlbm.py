@@ -127,7 +127,8 @@ def rlbm_workspace_bytes(specs, edf, storage, order=5):
 
 def rlbm_layout_tiles(specs, edf, storage, packed):
     """The tile work list (rows of domain, x0, y0, w) a handle of these domains
-    would walk: the plain 32 x 4 list, or the packed one of the FP64 and the mixed L1 steps."""
+    would walk: the plain 32 x 4 list, or the packed one of the FP64 and the mixed L1 steps
+    (w + 256: a packed tile of one warp)."""
     doms = make_domains(specs)
     cfg = rlbm_config(len(specs), doms, edf, storage, 5, None, 0, None)
     n = _check(load().rlbm_layout_tiles(ctypes.byref(cfg), int(packed), None, 0))
