@@ -136,8 +136,10 @@ size_t rlbm_workspace_bytes(const rlbm_config *config);
  * 32 x 4 tiles (TMA-staged step, initialisers, read-outs), packed = 1
  * the list of the FP64 and the mixed L1 steps, where each domain's ragged last x block of
  * w <= 16 cells is one tile per 4 * (32 / w) rows, a warp covering 32 / w rows
- * of w cells, or, in mixed launches of one wave, one tile per 32 / w rows of which only
- * the first warp works, listed with w + 256. Writes up to max_tiles quadruples (domain, x0, y0, w) to `out`
+ * of w cells. A mixed launch whose list stays within one wave of blocks (608, or 760 for the
+ * FP32 storages without walls and zero-gradient sides, blocks at most 6 wide) has instead
+ * one tile per 32 / w rows, of which only the first warp works, listed with w + 256.
+ * Writes up to max_tiles quadruples (domain, x0, y0, w) to `out`
  * (host, int[4 * max_tiles]; may be null) and returns the number of tiles, or
  * RLBM_E_ARG for an invalid configuration. */
 int rlbm_layout_tiles(const rlbm_config *config, int packed, int *out, int max_tiles);

@@ -18,12 +18,30 @@ using namespace rlbm;
 namespace {
 
 constexpr size_t kAlign = 256;
-// A mixed launch of at most this many tiles is one wave (4 blocks on each of 152 SMs) and
-// lasts as long as its longest block. There the packed tiles go one warp to a block
-// (kOneWarp): a packed warp's accesses touch up to 32 rows, so four in one SM were the
-// pole (129^2 domain: 17.4 us a step, 128^2: 5.6 us). Larger launches keep whole
-// tiles, whose fourth of the blocks matters more.
-constexpr size_t kOneWaveTiles = 4 * 152;
+// A mixed launch of one wave lasts as long as its longest block. Where the packed tiles at
+// one warp to a block (kOneWarp) stay within the wave, they go so: a packed warp's accesses
+// touch up to 32 rows, so four in one SM were the pole (FP32 deviations, us a step, whole
+// packed tiles / one warp a block: 129^2 17.7 / 8.8, 33 x 1600 21.5 / 11.3, 3 x 1500 8.5 /
+// 7.1, 16 x 600 5.7 / 5.6). A launch that would leave the wave keeps whole tiles, whose
+// fourth of the blocks matters more (16 x 4096, 512 or 2,048 blocks: 8.4 / 15.5; 48 x 1024
+// 7.7 / 11.0; 4 x 19000 24.0 / 40.7; 600 domains of 8 x 10 8.0 / 15.8; only at w = 1 the
+// other way by a tenth, 1 x 41600 111 / 96).
+// The wave: 152 SMs, 4 blocks each. The FP32 storages without halo work fit 5; the fifth
+// counts where the packed blocks are narrow and the pole long (700 blocks, whole / one warp:
+// 3 x 7000 11.5 / 9.6, 35 x 2000 15.4 / 11.1; at 12 cells 44 x 933 7.7 / 9.4).
+constexpr size_t kSms = 152;
+constexpr int kNarrowW = 6;  // 102 x 736, 700 blocks: 12.9 / 10.9; 40 x 1400: 8.5 / 10.7
+
+size_t one_wave_blocks(const rlbm_config* c, const std::vector<Tile>& packed) {
+  bool fifth = c->storage == RLBM_F32 || c->storage == RLBM_F32DEV;
+  for (int i = 0; i < c->ndomains; ++i) {
+    const rlbm_domain& d = c->domains[i];
+    for (int b : {d.bc_xlo, d.bc_xhi, d.bc_ylo, d.bc_yhi}) fifth = fifth && !bc_writes_halo(b);
+  }
+  for (const Tile& t : packed) fifth = fifth && t.w <= kNarrowW;
+  return (fifth ? 5 : 4) * kSms;
+}
+
 constexpr int kChunkPairs = 16;  // a chunk graph holds 2 * kChunkPairs steps
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -46,7 +64,7 @@ struct Layout {
   std::vector<DomDev> dd;
   std::vector<Tile> tiles;   // kTileW x kTileH tiles: the TMA-staged step, initialisers, read-outs
   std::vector<Tile> ptiles;  // the same with each domain's ragged last x block packed (Tile::w)
-  std::vector<Tile> otiles;  // that at one warp per packed tile (see kOneWaveTiles), or empty
+  std::vector<Tile> otiles;  // that at one warp per packed tile (see one_wave_blocks), or empty
   // what the FP64 and the mixed L1 step walk
   const std::vector<Tile>& stiles() const { return otiles.empty() ? ptiles : otiles; }
 };
@@ -144,7 +162,8 @@ void make_layout(const rlbm_config* c, Layout& L) {
     }
   }
   L.otiles.clear();
-  if (c->storage != RLBM_F64 && L.ptiles.size() <= kOneWaveTiles)
+  const size_t wave = one_wave_blocks(c, L.ptiles);
+  if (c->storage != RLBM_F64 && L.ptiles.size() <= wave) {
     for (const Tile& t : L.ptiles) {
       const int r = packed_rows_per_warp(t.w);
       if (!t.w) L.otiles.push_back(t);
@@ -152,6 +171,8 @@ void make_layout(const rlbm_config* c, Layout& L) {
         for (int k = 0; k < kTileH && t.y0 + k * r < L.dd[t.dom].ny; ++k)
           L.otiles.push_back(Tile{t.dom, t.x0, t.y0 + k * r, t.w + kOneWarp});
     }
+    if (L.otiles.size() > wave) L.otiles.clear();
+  }
   L.pop_elems = off;
   L.pop_bytes = align_up(off * es, kAlign);
   size_t b = 0;
