@@ -100,10 +100,14 @@ __device__ __forceinline__ double widen_f64(float x) {
 // ------------------------------------------------ FP64 divide and square root
 // GB300 issues one FP64 warp instruction per SM sub-partition every 64 clocks, so a
 // reciprocal or a root costs what its FP64 instructions cost. Both start from the
-// FP32 unit's value (about 23 bits) and take one step of a third-order (Halley)
-// iteration in FP64: with e = 1 - x r, 1/x = r (1 + e + e^2 + ...), and with
-// e = 1 - x r^2, 1/sqrt(x) = r (1 + e/2 + 3 e^2/8 + ...); the terms left out are
-// below 2^-64. Outside the FP32 range they fall back to the compiler's own.
+// FP32 unit's value r (about 23 bits) and take three terms of a series in FP64: with
+// e = 1 - x r, 1/x = r (1 + e + e^2 + ...), and with e = 1 - x r^2, 1/sqrt(x) =
+// r (1 + e/2 + 3 e^2/8 + ...); the terms left out are below 2^-64. Largest relative
+// errors: rcp64 half an ulp, as the division; rsqrt64 1.5 * 2^-53, where 1 / sqrt(x)
+// rounds twice. Outside the FP32 range they fall back to the compiler's own. (A quotient
+// a * rcp64(b) rounds once more than a / b. With the residual applied, as the division
+// has it, the read-out temperature's error is the same to 1 % and the FP64 steps take
+// 0.4 % longer: not taken.)
 __device__ __forceinline__ double rcp64(double x) {
   const float xf = cut_f32(x);
   if (!(fabsf(xf) > 1e-30f && fabsf(xf) < 1e30f)) return 1.0 / x;
