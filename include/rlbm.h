@@ -144,8 +144,8 @@ size_t rlbm_workspace_bytes(const rlbm_config *config);
  * RLBM_E_ARG for an invalid configuration. */
 int rlbm_layout_tiles(const rlbm_config *config, int packed, int *out, int max_tiles);
 
-/* Create a handle over the caller's workspace. Copies the descriptors; uploads
- * the tables; does not initialise populations. *out = NULL on error. */
+/* Create a handle over the caller's workspace. Copies the descriptors and uploads
+ * the tile lists; does not initialise populations. *out = NULL on error. */
 int rlbm_create(const rlbm_config *config, rlbm_handle *out);
 
 /* Set domain `domain` to the equilibrium f = f^eq of the given fields (time 0;

@@ -247,7 +247,6 @@ cudaError_t launch_step(rlbm_ctx* h, int from) {
   const size_t per = (size_t)h->ndom * kTensorMapBytes;
   const bool tma = h->d_tmaps && h->kernel == RLBM_KERNEL_TMA;
   a.tmaps = tma ? h->d_tmaps + (size_t)from * per : nullptr;
-  a.variant = h->kernel;
   a.wait_ns = h->wait_ns;
   a.halo = h->halo;
   a.images = 0;

@@ -92,7 +92,7 @@ constexpr int kTileW = 32, kTileH = RLBM_TILE_H;
 // (32 / w) * w on idle), so the tile spans kTileH * (32 / w) rows.
 // With kOneWarp added to w only warp 0 of the tile works: a launch of one wave is as
 // long as its longest block, and the accesses of a packed warp take a sector per
-// row, so there each packed warp gets a block of its own (see make_layout).
+// row, so there each packed warp gets a block of its own (see one_wave_blocks).
 struct Tile {
   int dom, x0, y0, w;
 };
@@ -122,8 +122,8 @@ struct StepArgs {
   const void* fin;        // population copy read (post-collision, with halo)
   void* fout;             // population copy written
   unsigned* status;       // OR of per-cell status bits
-  const void* tmaps;      // TMA load descriptors of fin, one per domain (kTensorMapBytes each), or null
-  int variant;            // mixed step kernel (RLBM_KERNEL_*); the FP64 step has one
+  const void* tmaps;      // TMA load descriptors of fin, one per domain (kTensorMapBytes each), for
+                          // the TMA-staged step, or null
   int halo;               // halo work of the launch: 0 none (every side periodic or exchanged),
                           // 1 wall equilibria only, 2 also zero-gradient copies, 3 also velocity
                           // walls (FP64 storage only)

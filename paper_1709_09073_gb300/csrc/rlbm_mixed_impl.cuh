@@ -1244,6 +1244,7 @@ static cudaError_t prepare_mixed_t() {
   return cudaFuncSetAttribute(k_step_mixed<EDF, S, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemF);
 }
 
+// Shared-memory limits of a storage's kernels.
 template <class S>
 static cudaError_t prepare_s() {
   cudaError_t e;
@@ -1296,15 +1297,9 @@ struct MixedUnit {
   cudaError_t (*copy)(const CopyArgs& a, cudaStream_t s);
 };
 
-// Shared-memory limits of this unit's kernels.
-template <class S>
-static cudaError_t prepare_unit() {
-  return prepare_s<S>();
-}
-
 template <class S>
 constexpr MixedUnit mixed_unit() {
-  return MixedUnit{&prepare_unit<S>, &step_s<S>, &launch_init_mixed_t<S>, &launch_fields_mixed_t<S>,
+  return MixedUnit{&prepare_s<S>, &step_s<S>, &launch_init_mixed_t<S>, &launch_fields_mixed_t<S>,
                    &launch_copy_t<S>};
 }
 

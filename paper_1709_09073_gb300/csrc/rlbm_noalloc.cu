@@ -182,7 +182,6 @@ extern "C" int rlbm_step_noalloc(const rlbm_domain* domain, int edf, int nsteps,
     a.fout = pop[1 - cur];
     a.status = d_status;
     a.tmaps = nullptr;
-    a.variant = 0;
     a.wait_ns = 0;
     a.halo = 3;  // any side
     a.images = 1;  // f_out holds the whole halo
