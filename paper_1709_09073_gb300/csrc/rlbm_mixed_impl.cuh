@@ -1109,7 +1109,7 @@ cudaError_t launch_fields_mixed_t(int edf, const FieldsArgs& a, int nx, int ny, 
 }
 
 // f = f^eq of the given fields in a mixed storage (time zero), halo included:
-// the collision's FP32 equilibrium deviations (dz_moments, dfeq_shell, with the
+// the collision's FP32 equilibrium deviations (dz_moments, dfeq_pair, with the
 // tables' conserved-moment defects removed) from the FP64 input fields. Its
 // rounding is that of every collision of the mixed step, and it runs on the
 // FP32 pipe (an FP64 initialiser costs as much as ten mixed steps on GB300).
